@@ -896,6 +896,19 @@ void tune_store(const sbqa_problem *p, const TuneResult &r) {
   g_tune[tune_key(p)] = r;
 }
 
+// Clears the f buffers before a trial launch of a persistent CSR solver: the
+// buffer such a launch starts from holds plain codes (or positions below 2),
+// and a trial runs on recycled memory.
+cudaError_t clear_f(sbqa_problem *p) {
+  const size_t NC = size_t(p->n) * p->Cp;
+  if (p->ballistic()) {
+    const cudaError_t e = cudaMemsetAsync(p->d_Fx0.p, 0, NC * sizeof(float), p->stream);
+    return e != cudaSuccess ? e : cudaMemsetAsync(p->d_Fx1.p, 0, NC * sizeof(float), p->stream);
+  }
+  const cudaError_t e = cudaMemsetAsync(p->d_F0.p, 0, NC, p->stream);
+  return e != cudaSuccess ? e : cudaMemsetAsync(p->d_F1.p, 0, NC, p->stream);
+}
+
 // The ballistic form has one per-step kernel and, where the items fit the
 // cache, the persistent solver: kernel_select 1 keeps the per-step kernel, 2
 // the persistent solver, 0 times both (a few steps each) and keeps the faster.
@@ -929,8 +942,11 @@ int autotune_csr_bsb(sbqa_problem *p) {
       cudaEvent_t e0, e1;
       SBQA_CUDA(cudaEventCreate(&e0));
       SBQA_CUDA(cudaEventCreate(&e1));
-      cudaError_t e = launch_solve_csr_persistent_bsb(s, J, p->tables, 0, std::min(p->S, 4), p->d_bar.p, p->d_err.p,
-                                                      p->persist_blocks, p->stream);
+      cudaError_t e = clear_f(p);
+      if (e == cudaSuccess)
+        e = launch_solve_csr_persistent_bsb(s, J, p->tables, 0, std::min(p->S, 4), p->d_bar.p, p->d_err.p,
+                                            p->persist_blocks, p->stream);
+      if (e == cudaSuccess) e = clear_f(p);
       if (e == cudaSuccess) e = cudaEventRecord(e0, p->stream);
       if (e == cudaSuccess)
         e = launch_solve_csr_persistent_bsb(s, J, p->tables, 0, steps, p->d_bar.p, p->d_err.p, p->persist_blocks,
@@ -1022,8 +1038,10 @@ int autotune_csr(sbqa_problem *p) {
   } else if (p->prm.kernel_select == 0 && p->S > 0 && p->persistent_ok()) {
     SBQA_CUDA(p->d_bar.alloc(persistent_barrier_words()));
     const int steps = std::min(p->S, 64);
+    SBQA_CUDA(clear_f(p));
     SBQA_CUDA(launch_solve_csr_persistent(s, J, p->tables, 0, std::min(p->S, 4), p->d_bar.p, p->d_err.p,
                                           p->persist_blocks, p->persist_mode(), p->stream));
+    SBQA_CUDA(clear_f(p));
     SBQA_CUDA(cudaEventRecord(e0, p->stream));
     SBQA_CUDA(launch_solve_csr_persistent(s, J, p->tables, 0, steps, p->d_bar.p, p->d_err.p, p->persist_blocks,
                                           p->persist_mode(), p->stream));
@@ -1780,6 +1798,7 @@ int sbqa_run_begin(sbqa_problem *p, int32_t steps, int32_t P, int32_t R, uint64_
   if (rc != SBQA_OK) return rc;
   DeviceGuard g(p->device);
   p->small_path = false;
+  p->wide_x = false;
   p->stream = static_cast<cudaStream_t>(stream);
   p->begun = p->finished = false;
   rc = p->dense ? prepare_dense_values(p, p->prm.precision) : prepare_sparse_values(p, p->prm.precision);
@@ -1985,6 +2004,8 @@ int sbqa_set_state(sbqa_problem *p, const float *x, const float *y, int32_t step
         by[size_t(i) * p->Cp + c] = y[o + i];
       }
     }
+  p->wide_x = false;
+  for (float v : bx) p->wide_x = p->wide_x || !(std::fabs(v) < 2.f);
   SBQA_CUDA(cudaMemcpy(p->d_x.p, bx.data(), NC * sizeof(float), cudaMemcpyHostToDevice));
   SBQA_CUDA(cudaMemcpy(p->d_y.p, by.data(), NC * sizeof(float), cudaMemcpyHostToDevice));
   const double tau = p->S > 0 ? double(step_done) / double(p->S) : 0.0;

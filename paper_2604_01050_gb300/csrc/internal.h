@@ -69,6 +69,7 @@ struct CsrView {
   const int32_t *ell_col;
   const float *ell_val;
   const int32_t *ell_meta;
+  int max_degree;
 };
 
 constexpr int kEllSlots = 8;
@@ -106,17 +107,30 @@ struct BestView {
 // returns code.
 int set_error(int code, const std::string &msg);
 
-// All steps of a +-1 CSR run batch in one cooperative launch with a bounded
-// grid barrier between steps (solve_persistent.cu).
+// All steps of a CSR run batch in one cooperative launch.  Two forms: with as
+// much of the state on the chip as fits, rows waiting on their neighbours'
+// codes (solve_persistent.cu); and with the state streamed and a grid barrier
+// per step (solve_streaming.cu).  blocks: persistent_blocks(); bar:
+// grid_barrier_words() counters.
 int persistent_blocks();
-int persistent_barrier_words();  // size of the barrier counter buffer
-// 0: not eligible; 1: items cached per warp; 2: whole rows cached per warp
-// (force_rows: rows whenever they fit); 3: items, as many cached per warp as
-// fit and the rest read from the ELL arrays every step (ell: the ELL form
-// exists); kind = the CSR value kind
+// 0: not eligible; kPersistResident: the first form; else the streaming form
+// -- 1: items cached per warp; 2: whole rows cached per warp (force_rows: rows
+// whenever they fit); 3: items, as many cached per warp as fit and the rest
+// read from the ELL arrays every step (ell: the ELL form exists); kind = the
+// CSR value kind
+constexpr int kPersistResident = 4;
 int persistent_mode(int N, int Cp, int max_degree, int kind, int blocks, bool force_rows, bool ell);
 cudaError_t launch_solve_csr_persistent(const StateView &s, const CsrView &J, const StepTables &t, int n_begin,
                                         int n_end, unsigned *bar, int *err, int blocks, int mode, cudaStream_t st);
+constexpr int kStreamBlocksPerSm = 4;
+bool streaming_fits();
+int streaming_mode(int N, int Cp, int max_degree, int kind, int blocks, bool force_rows, bool ell);
+cudaError_t launch_solve_csr_streaming(const StateView &s, const CsrView &J, const StepTables &t, int n_begin,
+                                       int n_end, unsigned *bar, int *err, int blocks, int mode, cudaStream_t st);
+int persistent_barrier_words();
+bool streaming_bsb_ok(int N, int Cp, int max_degree, int kind, int blocks);
+cudaError_t launch_solve_csr_streaming_bsb(const StateView &s, const CsrView &J, const StepTables &t, int n_begin,
+                                           int n_end, unsigned *bar, int *err, int blocks, cudaStream_t st);
 // The ballistic form f(x) = x in one cooperative launch (items of 128 columns
 // cached per warp; f buffers Fx in FP32): eligible when the items fit the
 // cache (persistent_bsb_ok); results equal launch_step_csr_bsb bit for bit.

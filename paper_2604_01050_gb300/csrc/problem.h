@@ -193,8 +193,9 @@ struct sbqa_problem {
   float variant_ms[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
   bool use_persistent = false;  // autotuner: one cooperative launch for all steps
   float persistent_ms = 0.f;    // its timing per step
+  bool wide_x = false;  // sbqa_set_state gave some |x| >= 2 or NaN: ballistic runs stay on the per-step kernel
   int persist_blocks = 0;
-  sbqa::DevBuf<unsigned> d_bar;  // grid barrier counter of the persistent kernel
+  sbqa::DevBuf<unsigned> d_bar;  // grid barrier counters of the streaming form
   int csr_variant_cp = -1, csr_variant_kind = -1, csr_variant_select = -1;
   // dense tcgen05: per-step kernel or the persistent solver (autotuned per Cp and kernel_select)
   bool use_tc_persistent = false;
@@ -294,7 +295,7 @@ struct sbqa_problem {
 
   bool persistent_ok() const {
     if (dense) return false;
-    if (ballistic()) return sbqa::persistent_bsb_ok(n, Cp, max_degree, kind, persist_blocks);
+    if (ballistic()) return !wide_x && sbqa::persistent_bsb_ok(n, Cp, max_degree, kind, persist_blocks);
     return persist_mode() != 0;
   }
 
@@ -315,7 +316,7 @@ struct sbqa_problem {
   }
   CsrView csr() const {
     CsrView v;
-    v.row_ptr = d_row_ptr.p; v.h = d_h.p; v.kind = kind; v.npos = d_npos.p;
+    v.row_ptr = d_row_ptr.p; v.h = d_h.p; v.kind = kind; v.npos = d_npos.p; v.max_degree = max_degree;
     v.col = kind == VAL_PM1 ? d_col_pm1.p : d_col.p;
     v.val = kind == VAL_F32 ? static_cast<const void *>(d_val_f32.p)
                             : static_cast<const void *>(d_val_bf16.p);

@@ -1,338 +1,634 @@
 // solve_persistent.cu -- all steps of a CSR run batch in one cooperative launch.
 //
-// For rows of degree <= 8 (+-1, FP32 or BF16 couplings).  The grid is exactly
-// as large as can be co-resident; every warp owns fixed work items (spin row,
-// chunk of 32 W replica columns, W = 4 or 8) for the whole anneal --
-// individual items, or whole rows with all their chunks when the items
-// outnumber the cache.  Before the first step a warp copies the column
-// indices (and signs or values) of its rows into shared memory, so a step
-// needs no index loads: per item it gathers the f codes of the (at most 8)
-// neighbours and the x, y of its columns, sums (same arithmetic and order as
-// k_step_csr), updates and writes x, y and the next codes.  The codes
-// written by other blocks are read through L2 (ld.global.cg), never the
-// non-coherent path.  Between steps all blocks meet at a grid barrier; the
-// wait is bounded (1 s, or at once when another block has already failed):
-// a block that gives up records an error and stops stepping, so a broken
-// grid ends with a status the host reads.
+// For rows of degree <= 8 (+-1, FP32 or BF16 couplings).  One block of 32
+// warps per SM; every warp owns fixed work items (spin row, 128 or 256
+// replica columns) for the whole launch -- individual items, or whole rows
+// with all their chunks when the items outnumber the cache.  A pass is what
+// the warp works on at a time: one 256-column item, or two 128-column ones on
+// its half warps (8 columns per lane either way).
+//
+// What a launch reads from memory more than once it keeps on the SM:
+//   neighbour lists (columns, signs or values, degrees) in shared memory;
+//   x and y of a warp's first passes in tensor memory (the block takes all
+//   512 TMEM columns; 64 per warp hold 4 passes of 8 + 8 values per lane) and
+//   of the next passes in the shared memory the lists leave (2 KB each).
+// Passes past those keep x and y in global memory, so a launch of any size
+// streams only the part of its state that does not fit the chip.  The 152
+// SMs hold 38 MB of state in TMEM and up to 31 MB in shared memory: all of the
+// 67 MB of the L = 16 lattice with R*P = 2048, 58 % of the 102 MB of N = 10^5
+// with R*P = 128.  Between SMs only the one-byte f codes move, through L2
+// (ld.global.cg: other blocks wrote them).
+//
+// What bounds a pass then is the ALU pipe (compares, selects, logic, byte
+// permutes at half rate: about 150 a pass) and the latency of the gathers; 24
+// warps of 80 registers were faster than 32 of 64, which spill (lattice L = 16
+// 13.3 against 16.1 us per step), and one 2 KB state slot per warp faster than
+// more, which take the L1 the gathers pass through (14.5 with three, 17.4 with
+// four).  us per step, before (the streaming form) and with this kernel:
+//   lattice L = 16, R*P = 2048     24.0 -> 13.3    random graph N = 10^5,
+//   lattice L = 10, R*P = 1024      4.9 ->  3.1    R*P = 128, BF16 46.8 -> 27.8
+//   lattice L = 24, R*P = 2048     81.9 -> 70.2    N = 3000 3.0 -> 2.0
+//   ballistic L = 16 36.6 -> 32.0, L = 12, R*P = 512 5.6 -> 3.8, N = 10^5 61.8 -> 55.3
+//
+// Per pass a warp gathers the codes of the (at most 8) neighbours, sums (same
+// arithmetic and order as k_step_csr), updates and writes the next codes.
+//
+// Steps are not separated by a grid barrier: every f code carries one bit of
+// its generation, and a warp that gathers a code of the generation before
+// reads it again until the new one has arrived.  The f buffers alternate by
+// step parity, so a buffer's generation is (steps since the launch began + 1)
+// / 2 mod 2, and the bit tells the codes of step n from those of step n - 2
+// (0 in the buffer the launch starts from, and in the other one, which the
+// launch clears first; the host keeps ballistic states with |x| >= 2, whose
+// bit would read as 1, on the per-step kernel).  Overwriting is safe because the couplings are
+// symmetric: row i writes f_{n+1} over f_{n-1} only after it has read f_n of
+// all its neighbours, and a neighbour wrote its f_n after it had read f_{n-1}
+// of row i.  A code is its own message (one byte holds value and bit), so no
+// fence orders it behind anything else.  The grid is co-resident
+// (cooperative launch), so the lowest step always progresses.  A wait is
+// bounded (1 s, or at once when another warp has already failed): a warp that
+// gives up records an error and stops stepping, and the launch ends with a
+// status the host reads.
 #include <algorithm>
 #include <cstdlib>
 #include <type_traits>
 
-#include "grid_sync.cuh"
+#include "grid_sync.cuh"  // globaltimer_ns and the limits of a bounded wait
 #include "step_common.cuh"
+#include "tc_common.cuh"
 
 namespace sbqa {
 
 constexpr int kPersistMaxDeg = 8;
-constexpr size_t kPersistSmem = 46080;  // per block: under the 48 KB default with the static barrier flag
+constexpr int kPersistWarps = 24, kPersistThreads = 32 * kPersistWarps;
+constexpr int kPersistSmem = 225 * 1024;               // dynamic shared memory of a block
+constexpr int kWarpSmem = kPersistSmem / kPersistWarps;  // 9600 bytes per warp
+constexpr int kSlotBytes = 2048;                       // x, y of one pass: 16 floats x 32 lanes
+constexpr uint32_t kPersistTmem = 512;                 // the block takes all TMEM columns of its SM
+constexpr int kMaxSlots = 1;                           // state slots per warp: what shared memory takes, L1 lacks
+// Passes per warp; run batches with more take the streaming form (30 passes, L
+// = 24: 70 us per step against 82 there; 72, L = 32: 183 there)
+constexpr int kMaxPasses = 40;
+static_assert(2 * kMaxPasses * 76 + kSlotBytes <= kWarpSmem, "lists and state slots fit a warp's shared memory");
+constexpr int kTmemPasses = 5;                         // x, y of 5 passes
+constexpr int kWarpTmem = 80;                          // TMEM columns per warp: 6 warps share a lane quarter
+static_assert(kPersistWarps / 4 * kWarpTmem <= 512 && 16 * kTmemPasses <= kWarpTmem, "TMEM columns");
+static_assert(kWarpSmem % 16 == 0, "warp regions hold 16-byte vectors");
 
 struct PersistArgs {
   StateView s;
-  const int32_t *row_ptr, *col, *npos;  // CSR (+-1: each row's +1 entries first)
-  const void *val;                      // FP32 or BF16 values (not +-1)
   const float *h;
-  // ELL form (mode 3: the items beyond a warp's cache read their neighbours here)
+  // ELL form of the couplings (rows of degree <= 8, the CSR kernels' entry order)
   const int32_t *ell_col, *ell_meta;
   const float *ell_val;
   StepTables t;
   int n_begin, n_end;
-  unsigned *bar;  // grid barrier counters (persistent_barrier_words(), zeroed before the launch)
   int *err;       // error flag
-  int skip_step;  // test hook: block 0 does not arrive at the barrier after this step (-1: never)
-  int cache_cap;  // items (or rows) a warp caches at most
+  int skip_step;  // test hook: block 0 does not publish the codes of this step (-1: never)
+  int degree;     // largest row degree: a pass reads 4, 6 or 8 slots
+  int cache_cap;  // items a warp holds at most
+  int slots;      // passes (ballistic form: items) whose state is kept in shared memory
+  int warp_smem;  // bytes of a warp's shared memory: its slots, then its cache
 };
 
-// Cache entries.  Items mode: one (row, chunk) item.  Rows mode: one row; its
-// index is gw + q * warps for the warp's q-th row.  (degree | +1 count << 8)
-// packed in degpos; values only for FP32 / BF16 couplings.
+// Bytes of one cached item: 8 columns, 8 values (signs as bytes for +-1), a
+// word of the degree and the sum of the signs, and (row, chunk).  Unused
+// slots name the row itself with weight 0, so that a pass reads the same
+// number of slots for every row without a test per slot.
+constexpr int entry_bytes(bool vals) { return 32 + (vals ? 32 : 8) + 4 + 8; }
+
+// A warp's cached neighbour lists, in arrays over its entries.
 template <bool VALS>
-struct ItemEntry {
-  int32_t col[kPersistMaxDeg];
-  int32_t row, chunk;
-  uint32_t degpos;
-};
-template <>
-struct ItemEntry<true> {
-  int32_t col[kPersistMaxDeg];
-  float val[kPersistMaxDeg];
-  int32_t row, chunk;
-  uint32_t degpos;
-};
-template <bool VALS>
-struct RowEntry {
-  int32_t col[kPersistMaxDeg];
-  uint32_t degpos;
-};
-template <>
-struct RowEntry<true> {
-  int32_t col[kPersistMaxDeg];
-  float val[kPersistMaxDeg];
-  uint32_t degpos;
+struct WarpCache {
+  int4 *cols;     // [2 cap]
+  float4 *vals;   // [2 cap]; +-1: int2 [cap] of signed bytes
+  int2 *item;     // [cap] (row, chunk)
+  uint32_t *meta;  // [cap] degree | (sum of signs) << 16
+  __device__ WarpCache(char *base, int cap) {
+    cols = reinterpret_cast<int4 *>(base);
+    base += 32 * cap;
+    vals = reinterpret_cast<float4 *>(base);
+    base += (VALS ? 32 : 8) * cap;
+    item = reinterpret_cast<int2 *>(base);
+    base += 8 * cap;
+    meta = reinterpret_cast<uint32_t *>(base);
+  }
+  // Fills entry q with row `row` (lanes 0-7 one slot each).
+  __device__ __forceinline__ void fill(const PersistArgs &a, int q, int row, int chunk, int lane) const {
+    const int2 m = __ldg(reinterpret_cast<const int2 *>(a.ell_meta) + row);  // (degree, +1 count)
+    if (lane < kPersistMaxDeg) {
+      const bool used = lane < m.x;
+      reinterpret_cast<int32_t *>(cols)[8 * q + lane] =
+          used ? __ldg(a.ell_col + size_t(row) * kPersistMaxDeg + lane) : row;
+      if constexpr (VALS)
+        reinterpret_cast<float *>(vals)[8 * q + lane] =
+            used ? __ldg(a.ell_val + size_t(row) * kPersistMaxDeg + lane) : 0.f;
+      else
+        reinterpret_cast<int8_t *>(vals)[8 * q + lane] = used ? (lane < m.y ? 1 : -1) : 0;
+    } else if (lane == kPersistMaxDeg) {
+      meta[q] = uint32_t(m.x) | (uint32_t(2 * m.y - m.x) << 16);
+      item[q] = make_int2(row, chunk);
+    }
+  }
 };
 
-template <bool ROWS, bool VALS>
-struct Cache {
-  using Entry = typename std::conditional<ROWS, RowEntry<VALS>, ItemEntry<VALS>>::type;
-  static constexpr int kPerWarp = int(kPersistSmem / 8 / sizeof(Entry));
-};
-
-// W bytes of f codes (one 4- or 8-byte load through L2: other blocks wrote
-// these codes in this launch).
-template <int W>
-struct Codes;
-template <>
-struct Codes<4> {
-  uint32_t w[1];
-  __device__ __forceinline__ void load(const uint8_t *p) { w[0] = __ldcg(reinterpret_cast<const uint32_t *>(p)); }
-  __device__ __forceinline__ void zero(uint32_t z) { w[0] = z; }
-};
-template <>
-struct Codes<8> {
+// f codes (8 bytes) and positions (16 bytes) that other SMs write in this
+// launch, through L2; volatile, so that a wait reads them again.
+struct Codes8 {
   uint32_t w[2];
   __device__ __forceinline__ void load(const uint8_t *p) {
-    const uint2 v = __ldcg(reinterpret_cast<const uint2 *>(p));
-    w[0] = v.x;
-    w[1] = v.y;
+    asm volatile("ld.relaxed.gpu.global.v2.u32 {%0, %1}, [%2];" : "=r"(w[0]), "=r"(w[1]) : "l"(p) : "memory");
   }
-  __device__ __forceinline__ void zero(uint32_t z) { w[0] = w[1] = z; }
+};
+__device__ __forceinline__ void publish(uint8_t *p, uint32_t a, uint32_t b) {
+  asm volatile("st.relaxed.gpu.global.v2.u32 [%0], {%1, %2};" ::"l"(p), "r"(a), "r"(b) : "memory");
+}
+struct Pos4 {
+  uint32_t w[4];
+  __device__ __forceinline__ void load(const float *p) {
+    asm volatile("ld.relaxed.gpu.global.v4.u32 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3])
+                 : "l"(p)
+                 : "memory");
+  }
 };
 
-// One item: x, y of the lane's W columns and the f codes of the row's
-// neighbours for those columns (issued together), the coupling sums (+-1:
-// packed code sums per sign; otherwise FP32 FMAs in entry order, as
-// k_step_csr), the update and the stores.
-// LPI lanes own one item of LPI * W columns: the whole warp (32), or half of
-// it (16: the warp works on two items at once, lanes 16-31 on the second;
-// act = false leaves a half without an item idle but in the shuffles).
-template <int P, int KIND, int W, bool GEN, int LPI = 32>
-__device__ __forceinline__ void persist_item(const PersistArgs &a, int i, int chunk, const int32_t *col,
-                                             const float *val, uint32_t degpos, const uint8_t *Fin, uint8_t *Fout,
-                                             float ka, float dnext, int n, int lane, bool act = true) {
-  const StateView &s = a.s;
-  const int deg = act ? int(degpos & 0xffu) : 0, npos = int(degpos >> 8);
-  const int c0 = chunk * LPI * W + (lane % LPI) * W;
-  const size_t off = size_t(i) * s.Cp + c0;
-  float xs[W], ys[W];
-#pragma unroll
-  for (int u = 0; u < W / 4; ++u) {
-    const float4 xa = *reinterpret_cast<const float4 *>(s.x + off + 4 * u);
-    const float4 ya = *reinterpret_cast<const float4 *>(s.y + off + 4 * u);
-    xs[4 * u] = xa.x; xs[4 * u + 1] = xa.y; xs[4 * u + 2] = xa.z; xs[4 * u + 3] = xa.w;
-    ys[4 * u] = ya.x; ys[4 * u + 1] = ya.y; ys[4 * u + 2] = ya.z; ys[4 * u + 3] = ya.w;
-  }
-  Codes<W> f[kPersistMaxDeg];
-#pragma unroll
-  for (int e = 0; e < kPersistMaxDeg; ++e) {
-    if (e < deg) f[e].load(Fin + size_t(col[e]) * s.Cp + c0);
-    else f[e].zero(KIND == VAL_PM1 ? 0u : kFZero4);
-  }
-  float G[W];
+// 8 consecutive floats, loaded where this stands in the program (a plain load
+// may be moved down to its use).
+__device__ __forceinline__ void load_row_now(const float *p, float (&v)[8]) {
+  asm volatile("ld.global.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]) : "l"(p));
+  asm volatile("ld.global.v4.f32 {%0, %1, %2, %3}, [%4];"
+               : "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7])
+               : "l"(p + 4));
+}
+
+// Generation bits: the top bit of every code byte; bit 30 of a position
+// (|x| <= 1 after an update, so its exponent leaves that bit 0).
+constexpr uint32_t kTagCodes = 0x80808080u, kTagPos = 0x40000000u;
+// the bit of step n's codes in a launch that began at step n0 (0 for n = n0)
+__device__ __forceinline__ uint32_t tag_of(int n, int n0, uint32_t bits) { return ((n - n0 + 1) & 2) ? bits : 0u; }
+
+// Whether the bounded wait that has read its entries `it` times gives up (looked
+// at every 16th time; t0 = 0 before); records the error then.
+__device__ __forceinline__ bool wait_over(unsigned it, uint64_t &t0, int *err) {
+  if ((it & 15) != 15) return false;
+  const uint64_t now = globaltimer_ns();
+  if (t0 == 0) t0 = now;
+  const bool over = now - t0 > kBarrierTimeoutNs || it > kBarrierSpins || *(volatile int *)err != 0;
+  if (!__any_sync(0xffffffffu, over)) return false;
+  if ((threadIdx.x & 31) == 0) atomicCAS(err, 0, 4);
+  return true;
+}
+
+// Coupling sums of one pass from the gathered codes of the lane's 8 columns
+// (with their generation bits).  +-1: packed sums of sign * code -- integers
+// modulo 2^32, so the bits and the offset codes carry are taken out at the
+// end, in the low mantissa bits of 2^23 (exact); otherwise FP32 FMAs in entry
+// order, as k_step_csr, each code through the low mantissa bits of 2^23.
+// The integer multiply-adds and FP32 adds run on the FMA pipes: the ALU pipe,
+// which takes every compare, select, logic and byte-permute instruction at
+// half rate, is what bounds a pass.
+template <int KIND>
+__device__ __forceinline__ void sum_codes(const Codes8 (&f)[kPersistMaxDeg], uint32_t tag, const float4 *vals,
+                                          uint32_t meta, int slots, float (&G)[8]) {
   if constexpr (KIND == VAL_PM1) {
-    uint32_t ap[W / 4], am[W / 4];
+    const int2 sg = *reinterpret_cast<const int2 *>(vals);
+    const int sum = int(meta) >> 16;
+    // per byte: 64 + sum over entries of sign * code, between 48 and 80
+    uint32_t acc[2];
+    acc[0] = acc[1] = 0x40404040u - tag * uint32_t(sum);
+    auto add = [&](int e) {
+      const uint32_t b = uint32_t(e & 3), w = uint32_t(e < 4 ? sg.x : sg.y);
+      uint32_t sign;  // byte b, sign extended
+      asm("prmt.b32 %0, %1, 0, %2;" : "=r"(sign) : "r"(w), "r"(b | (0x888u | b * 0x111u) << 4));
+      acc[0] += sign * f[e].w[0];
+      acc[1] += sign * f[e].w[1];
+    };
 #pragma unroll
-    for (int q = 0; q < W / 4; ++q) ap[q] = am[q] = 0;
-#pragma unroll
-    for (int e = 0; e < kPersistMaxDeg; ++e) {
-      if (e < npos) {
-#pragma unroll
-        for (int q = 0; q < W / 4; ++q) ap[q] += f[e].w[q];
-      } else {
-#pragma unroll
-        for (int q = 0; q < W / 4; ++q) am[q] += f[e].w[q];
-      }
+    for (int e = 0; e < 4; ++e) add(e);
+    if (slots > 4) {
+      add(4);
+      add(5);
     }
-    const int bias = (deg - npos) - npos;  // codes carry f + 1; missing entries add 0
+    if (slots > 6) {
+      add(6);
+      add(7);
+    }
+    const float off = -8388608.f - float(64 + sum);
 #pragma unroll
-    for (int c = 0; c < W; ++c)
-      G[c] = float(int((ap[c / 4] >> (8 * (c % 4))) & 0xffu) - int((am[c / 4] >> (8 * (c % 4))) & 0xffu) + bias);
+    for (int c = 0; c < 8; c += 2) {
+      const uint32_t m0 = __byte_perm(acc[c / 4], 0x4B000000u, 0x7540u | uint32_t(c % 4));
+      const uint32_t m1 = __byte_perm(acc[c / 4], 0x4B000000u, 0x7540u | uint32_t(c % 4 + 1));
+      const float2 g = __fadd2_rn(make_float2(__uint_as_float(m0), __uint_as_float(m1)), make_float2(off, off));
+      G[c] = g.x;
+      G[c + 1] = g.y;
+    }
   } else {
 #pragma unroll
-    for (int c = 0; c < W; ++c) G[c] = 0.f;
+    for (int c = 0; c < 8; ++c) G[c] = 0.f;
+    const float off = tag ? -8388737.f : -8388609.f;  // -(2^23 + 1), and the generation bit
+    const float4 v = vals[0];
+    acc_codes_off<8>(G, v.x, f[0].w, off);
+    acc_codes_off<8>(G, v.y, f[1].w, off);
+    acc_codes_off<8>(G, v.z, f[2].w, off);
+    acc_codes_off<8>(G, v.w, f[3].w, off);
+    if (slots > 4) {
+      const float4 u = vals[1];
+      acc_codes_off<8>(G, u.x, f[4].w, off);
+      acc_codes_off<8>(G, u.y, f[5].w, off);
+      if (slots > 6) {
+        acc_codes_off<8>(G, u.z, f[6].w, off);
+        acc_codes_off<8>(G, u.w, f[7].w, off);
+      }
+    }
+  }
+}
+
+// Whether all gathered codes carry the generation bits of tag: the AND (bits
+// set) or the OR (bits clear) of their words.
+__device__ __forceinline__ bool codes_fresh(const Codes8 (&f)[kPersistMaxDeg], uint32_t tag, int slots) {
+  if (tag) {
+    uint32_t v = f[0].w[0] & f[0].w[1];
 #pragma unroll
-    for (int e = 0; e < kPersistMaxDeg; ++e) {
-      if (e < deg) {
-        const float w = val[e];
-        acc_codes<W>(G, w, f[e].w);
-      }
-    }
+    for (int e = 1; e < 4; ++e) v &= f[e].w[0] & f[e].w[1];
+    if (slots > 4) v &= f[4].w[0] & f[4].w[1] & f[5].w[0] & f[5].w[1];
+    if (slots > 6) v &= f[6].w[0] & f[6].w[1] & f[7].w[0] & f[7].w[1];
+    return (v & kTagCodes) == kTagCodes;
   }
-  // an idle half takes part in the ring shuffles only (a column past C stores nothing)
-  sb_updateW<P, W, GEN>(s, a.t, ka, dnext, n, i, act ? c0 : s.C, G, __ldg(a.h + i), xs, ys, Fout);
+  uint32_t v = f[0].w[0] | f[0].w[1];
+#pragma unroll
+  for (int e = 1; e < 4; ++e) v |= f[e].w[0] | f[e].w[1];
+  if (slots > 4) v |= f[4].w[0] | f[4].w[1] | f[5].w[0] | f[5].w[1];
+  if (slots > 6) v |= f[6].w[0] | f[6].w[1] | f[7].w[0] | f[7].w[1];
+  return (v & kTagCodes) == 0;
 }
 
-template <int KIND>
-__device__ __forceinline__ float entry_value(const PersistArgs &a, int e) {
-  if constexpr (KIND == VAL_F32) return static_cast<const float *>(a.val)[e];
-  else return __bfloat162float(static_cast<const __nv_bfloat16 *>(a.val)[e]);
-}
-
-// ROWS = false: warp items (row, chunk) cached; true: whole rows cached.
-// LPI = 16 (items mode, W = 8): a half warp per item of 128 columns, two
-// items per warp at a time -- twice the items in flight per warp and half the
-// per-item instructions of W = 4 on a whole warp, same arithmetic per column.
-template <int P, bool ROWS, int KIND, int W, int LPI = 32>
-__global__ void __launch_bounds__(256, 4) k_solve_csr_persistent(PersistArgs a) {
+// LPI = 32: passes of one 256-column item on the whole warp; 16: of two 128-column ones on half warps.
+template <int P, int KIND, int LPI>
+__global__ void __launch_bounds__(kPersistThreads, 1) k_solve_csr_persistent(PersistArgs a) {
   constexpr bool VALS = KIND != VAL_PM1;
-  using C = Cache<ROWS, VALS>;
-  using Entry = typename C::Entry;
-  extern __shared__ int32_t s_cache[];  // [8 warps][C::kPerWarp] entries
+  constexpr int IPW = 32 / LPI;  // items per pass
+  extern __shared__ __align__(16) char s_raw[];
+  __shared__ uint32_t s_tmem;
   const StateView &s = a.s;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int chunks = s.Cp / (LPI * W);
-  const int warps_total = gridDim.x * 8;
-  const int gw = blockIdx.x * 8 + warp;
-  Entry *mine = reinterpret_cast<Entry *>(s_cache) + warp * C::kPerWarp;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, sub = lane / LPI;
+  const int chunks = s.Cp / (LPI * 8);
+  const int warps_total = gridDim.x * kPersistWarps;
+  const int gw = blockIdx.x * kPersistWarps + warp;
+  char *mine = s_raw + warp * a.warp_smem;
+  float4 *state = reinterpret_cast<float4 *>(mine);  // [slots][x lo, x hi, y lo, y hi][lane]
+  const WarpCache<VALS> cache(mine + a.slots * kSlotBytes, a.cache_cap);
+  if (warp == 0) tc::tmem_alloc(&s_tmem, kPersistTmem);
   int my_count = 0;
-  const int n_units = ROWS ? s.N : s.N * chunks;
-  const int cap = C::kPerWarp < a.cache_cap ? C::kPerWarp : a.cache_cap;
-  for (int u = gw; u < n_units && my_count < cap; u += warps_total, ++my_count) {
-    if (lane == 0) {
-      const int row = ROWS ? u : u / chunks;
-      const int e0 = a.row_ptr[row], e1 = a.row_ptr[row + 1];
-      Entry &m = mine[my_count];
-      if constexpr (!ROWS) {
-        m.row = row;
-        m.chunk = u - row * chunks;
-      }
-      m.degpos = uint32_t(e1 - e0) | (uint32_t(KIND == VAL_PM1 ? a.npos[row] : e1 - e0) << 8);
-      for (int q = 0; q < kPersistMaxDeg; ++q) {
-        m.col[q] = q < e1 - e0 ? a.col[e0 + q] : 0;
-        if constexpr (VALS) m.val[q] = q < e1 - e0 ? entry_value<KIND>(a, e0 + q) : 0.f;
-      }
-    }
+  const int n_units = s.N * chunks;
+  for (int u = gw; u < n_units && my_count < a.cache_cap; u += warps_total, ++my_count) {
+    const int row = u / chunks;
+    cache.fill(a, my_count, row, u - row * chunks, lane);
   }
-  __syncwarp();
-  unsigned k = 0;
+  tc::tc_fence_before();
+  __syncthreads();
+  tc::tc_fence_after();
+  // TMEM columns of this warp: its 32 lanes of the quarter warp % 4
+  const uint32_t tm = s_tmem + (uint32_t(warp & 3) << 21) + uint32_t(warp >> 2) * kWarpTmem;
+  const int passes = (my_count + IPW - 1) / IPW;
+  const int resident = min(passes, kTmemPasses + a.slots);
+
+  // A pass: the entry, row and first column of this lane; live = false: a half warp without an
+  // item, or columns past C.
+  struct Pass {
+    int e, i, c0;
+    bool live;
+  };
+  auto locate = [&](int p) {
+    Pass t;
+    t.e = p * IPW + sub;
+    t.live = t.e < my_count;
+    if (!t.live) t.e = p * IPW;
+    const int2 it = cache.item[t.e];
+    t.i = it.x;
+    t.c0 = it.y * (LPI * 8) + (lane % LPI) * 8;
+    t.live = t.live && t.c0 < s.C;
+    return t;
+  };
+  auto put = [&](int p, const float (&xs)[8], const float (&ys)[8]) {
+    if (p < kTmemPasses) {
+      uint32_t r[16];
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        r[j] = __float_as_uint(xs[j]);
+        r[8 + j] = __float_as_uint(ys[j]);
+      }
+      tc::tmem_st_32x32b_x16(tm + uint32_t(p) * 16u, r);
+    } else {
+      float4 *q = state + (p - kTmemPasses) * 128 + lane;
+      q[0] = make_float4(xs[0], xs[1], xs[2], xs[3]);
+      q[32] = make_float4(xs[4], xs[5], xs[6], xs[7]);
+      q[64] = make_float4(ys[0], ys[1], ys[2], ys[3]);
+      q[96] = make_float4(ys[4], ys[5], ys[6], ys[7]);
+    }
+  };
+  auto get = [&](int p, float (&xs)[8], float (&ys)[8]) {
+    if (p < kTmemPasses) {
+      uint32_t r[16];
+      tc::tmem_ld_32x32b_x16_nowait(tm + uint32_t(p) * 16u, r);
+      tc::tmem_wait_ld();
+      tc::reg_fence_n(r);
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        xs[j] = __uint_as_float(r[j]);
+        ys[j] = __uint_as_float(r[8 + j]);
+      }
+    } else {
+      const float4 *q = state + (p - kTmemPasses) * 128 + lane;
+      const float4 x0 = q[0], x1 = q[32], y0 = q[64], y1 = q[96];
+      xs[0] = x0.x; xs[1] = x0.y; xs[2] = x0.z; xs[3] = x0.w; xs[4] = x1.x; xs[5] = x1.y; xs[6] = x1.z; xs[7] = x1.w;
+      ys[0] = y0.x; ys[1] = y0.y; ys[2] = y0.z; ys[3] = y0.w; ys[4] = y1.x; ys[5] = y1.y; ys[6] = y1.z; ys[7] = y1.w;
+    }
+  };
+  for (int p = 0; p < resident; ++p) {
+    const Pass t = locate(p);
+    float xs[8], ys[8];
+    load_row<8>(s.x + size_t(t.i) * s.Cp + t.c0, xs);
+    load_row<8>(s.y + size_t(t.i) * s.Cp + t.c0, ys);
+    put(p, xs, ys);
+  }
   // replica counts below the run width take the general ring (one form per launch)
   const bool gen = P > 2 && s.Pr != P;
-  for (int n = a.n_begin; n < a.n_end; ++n) {
-    const uint8_t *Fin = s.f_of(n);
-    uint8_t *Fout = s.f_of(n + 1);
+
+  // the codes of a row's neighbours at step n
+  auto gather = [&](Codes8 (&f)[kPersistMaxDeg], int n, const int4 *cols, int c0) {
+    const uint8_t *F = s.f_of(n) + c0;
+    const int4 ca = cols[0];
+    f[0].load(F + size_t(ca.x) * s.Cp);
+    f[1].load(F + size_t(ca.y) * s.Cp);
+    f[2].load(F + size_t(ca.z) * s.Cp);
+    f[3].load(F + size_t(ca.w) * s.Cp);
+    if (a.degree > 4) {
+      const int4 cb = cols[1];
+      f[4].load(F + size_t(cb.x) * s.Cp);
+      f[5].load(F + size_t(cb.y) * s.Cp);
+      if (a.degree > 6) {
+        f[6].load(F + size_t(cb.z) * s.Cp);
+        f[7].load(F + size_t(cb.w) * s.Cp);
+      }
+    }
+  };
+  // Gathers until all codes are of step n (lanes that are not live do not wait); false when the
+  // warp gave up.
+  auto fresh = [&](Codes8 (&f)[kPersistMaxDeg], int n, const int4 *cols, int c0, bool live, uint32_t tag) {
+    uint64_t t0 = 0;
+    for (unsigned it = 0;; ++it) {
+      if (!__any_sync(0xffffffffu, live && !codes_fresh(f, tag, a.degree))) return true;
+      if (n == a.n_begin) return true;  // the codes a launch starts from are complete whatever their bits
+      if (wait_over(it, t0, a.err)) return false;
+      gather(f, n, cols, c0);
+    }
+  };
+  // Update of one pass from its coupling sums; slot < 0: the state is in xs, ys and goes back to
+  // global memory, else it lives on the chip in that slot.
+  auto update = [&](int n, const Pass &t, int slot, const float (&G)[8], const float (&kj)[P >= 8 ? 1 : 8 / P],
+                    float hi, float ka, float dnext, float (&xs)[8], float (&ys)[8]) {
+    const size_t off = size_t(t.i) * s.Cp + t.c0;
+    if (slot >= 0) get(slot, xs, ys);
+    float xm[8], xp[8];
+    if (gen) ring_nb<P, 8, true>(xs, s.Pr, xm, xp);
+    else ring_nb<P, 8, false>(xs, s.Pr, xm, xp);
+    if (t.live) {
+      uint32_t code[2];
+      sb_advanceW<P, 8>(s.C, a.t.kc, a.t.kx, ka, dnext, kj, t.c0, G, hi, xm, xp, xs, ys, code);
+      // the codes a launch leaves carry no bit
+      const uint32_t next = n + 1 < a.n_end ? tag_of(n + 1, a.n_begin, kTagCodes) : 0u;
+      if (!(n == a.skip_step && blockIdx.x == 0)) publish(s.f_of(n + 1) + off, code[0] | next, code[1] | next);
+      if (slot < 0) {
+        store_row<8>(s.x + off, xs);
+        store_row<8>(s.y + off, ys);
+      }
+    }
+    __syncwarp();
+    if (slot >= 0) put(slot, xs, ys);
+  };
+
+  bool ok = true;
+  for (int n = a.n_begin; ok && n < a.n_end; ++n) {
     const float ka = __ldg(a.t.ka + n), dnext = __ldg(a.t.dl + n + 1);
-    for (int q = 0; q < my_count; ++q) {
-      const Entry &m = mine[q];
-      const float *val = nullptr;
-      if constexpr (VALS) val = m.val;
-      if constexpr (ROWS) {
-        for (int ch = 0; ch < chunks; ++ch) {
-          if (gen)
-            persist_item<P, KIND, W, true>(a, gw + q * warps_total, ch, m.col, val, m.degpos, Fin, Fout, ka, dnext,
-                                           n, lane);
-          else
-            persist_item<P, KIND, W, false>(a, gw + q * warps_total, ch, m.col, val, m.degpos, Fin, Fout, ka, dnext,
-                                            n, lane);
-        }
-      } else if constexpr (LPI == 32) {
-        if (gen)
-          persist_item<P, KIND, W, true>(a, m.row, m.chunk, m.col, val, m.degpos, Fin, Fout, ka, dnext, n, lane);
-        else
-          persist_item<P, KIND, W, false>(a, m.row, m.chunk, m.col, val, m.degpos, Fin, Fout, ka, dnext, n, lane);
-      } else {
-        // lanes 16-31 take the next entry (idle past the warp's last one)
-        const int qq = q + (lane >> 4);
-        const bool act = qq < my_count;
-        const Entry &mh = mine[act ? qq : q];
-        const float *valh = nullptr;
-        if constexpr (VALS) valh = mh.val;
-        if (gen)
-          persist_item<P, KIND, W, true, LPI>(a, mh.row, mh.chunk, mh.col, valh, mh.degpos, Fin, Fout, ka, dnext, n,
-                                              lane, act);
-        else
-          persist_item<P, KIND, W, false, LPI>(a, mh.row, mh.chunk, mh.col, valh, mh.degpos, Fin, Fout, ka, dnext,
-                                               n, lane, act);
-        ++q;  // two entries per pass
+    const float *kjn = a.t.kj + size_t(n) * a.t.R;
+    const uint32_t tag = tag_of(n, a.n_begin, kTagCodes);
+    tc::tmem_wait_st();  // the step before's stores into TMEM are complete
+    for (int p = 0; p < passes; ++p) {
+      const Pass t = locate(p);
+      float xs[8], ys[8], G[8], kj[P >= 8 ? 1 : 8 / P];
+      if (p >= resident) {
+        const size_t off = size_t(t.i) * s.Cp + t.c0;
+        load_row_now(s.x + off, xs);
+        load_row_now(s.y + off, ys);
       }
+      Codes8 f[kPersistMaxDeg];
+      const int4 *cols = cache.cols + 2 * t.e;
+      gather(f, n, cols, t.c0);
+      load_kj<P, 8>(kjn, s.C, t.c0, kj);
+      const float hi = __ldg(a.h + t.i);
+      if (!(ok = fresh(f, n, cols, t.c0, t.live, tag))) break;
+      sum_codes<KIND>(f, tag, VALS ? cache.vals + 2 * t.e : reinterpret_cast<const float4 *>(
+                                                                reinterpret_cast<const int2 *>(cache.vals) + t.e),
+                      cache.meta[t.e], a.degree, G);
+      update(n, t, p < resident ? p : -1, G, kj, hi, ka, dnext, xs, ys);
     }
-    if constexpr (!ROWS) {
-      // items past the warp's cache (mode 3): neighbours from the ELL arrays
-      for (int u0 = gw + my_count * warps_total; u0 < n_units; u0 += (32 / LPI) * warps_total) {
-        const int uh = u0 + (LPI == 16 ? (lane >> 4) * warps_total : 0);
-        const bool act = uh < n_units;
-        const int u = act ? uh : u0;
-        const int row = u / chunks, ch = u - row * chunks;
-        const int2 meta = __ldg(reinterpret_cast<const int2 *>(a.ell_meta) + row);
-        const uint32_t dp = uint32_t(meta.x) | (uint32_t(KIND == VAL_PM1 ? meta.y : meta.x) << 8);
-        const int32_t *colp = a.ell_col + size_t(row) * kPersistMaxDeg;
-        const float *valp = VALS ? a.ell_val + size_t(row) * kPersistMaxDeg : nullptr;
-        if (gen)
-          persist_item<P, KIND, W, true, LPI>(a, row, ch, colp, valp, dp, Fin, Fout, ka, dnext, n, lane, act);
-        else
-          persist_item<P, KIND, W, false, LPI>(a, row, ch, colp, valp, dp, Fin, Fout, ka, dnext, n, lane, act);
-      }
+  }
+  tc::tmem_wait_st();
+  for (int p = 0; p < resident; ++p) {  // the resident state back to global memory
+    const Pass t = locate(p);
+    float xs[8], ys[8];
+    get(p, xs, ys);
+    if (t.live) {
+      store_row<8>(s.x + size_t(t.i) * s.Cp + t.c0, xs);
+      store_row<8>(s.y + size_t(t.i) * s.Cp + t.c0, ys);
     }
-    if (!grid_barrier(a.bar, ++k, a.err, n == a.skip_step && blockIdx.x == 0)) break;
+  }
+  tc::tc_fence_before();
+  __syncthreads();
+  if (warp == 0) {
+    tc::tc_fence_after();
+    tc::tmem_dealloc(s_tmem, kPersistTmem);
   }
 }
 
 // The ballistic form f(x) = x (the bSB choice named in Sec. II A): the same
-// persistent scheme in items mode with items of 128 columns on whole warps
-// (4 columns per lane), gathering the neighbours' FP32 positions of the step
-// before (written by other blocks: read through L2).  The sum runs over the
-// row's eight cache slots in order, a zero weight and a zero position past the
-// degree -- the sequence of fused multiply-adds of k_step_csr_bsb -- and the
-// update is sb_update4_bsb, so results equal the per-step kernel bit for bit.
+// scheme with items of 128 columns on whole warps (4 columns per lane),
+// gathering the neighbours' FP32 positions of the step before (written by
+// other blocks: read through L2).  An item's own x is its entry of that f
+// buffer, so only y is separate state: it stays in TMEM for a warp's first 16
+// items and in shared memory for the next ones (512 bytes each), and x goes
+// to the state array once, after the last step.  The sum runs over the row's
+// cache slots in order, a zero weight past the degree -- the sequence of
+// fused multiply-adds of k_step_csr_bsb -- and the update is sb_advance4_bsb,
+// so results equal the per-step kernel bit for bit.
+constexpr int kTmemItemsBsb = 20, kSlotBytesBsb = 512;
+
 template <int P, int KIND>
-__global__ void __launch_bounds__(256, 4) k_solve_csr_persistent_bsb(PersistArgs a) {
+__global__ void __launch_bounds__(kPersistThreads, 1) k_solve_csr_persistent_bsb(PersistArgs a) {
   constexpr bool VALS = KIND != VAL_PM1;
-  using C = Cache<false, VALS>;
-  using Entry = typename C::Entry;
-  extern __shared__ int32_t s_cache[];
+  extern __shared__ __align__(16) char s_raw[];
+  __shared__ uint32_t s_tmem;
   const StateView &s = a.s;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int chunks = s.Cp / kColsPerWarp;
-  const int warps_total = gridDim.x * 8;
-  const int gw = blockIdx.x * 8 + warp;
-  Entry *mine = reinterpret_cast<Entry *>(s_cache) + warp * C::kPerWarp;
+  const int warps_total = gridDim.x * kPersistWarps;
+  const int gw = blockIdx.x * kPersistWarps + warp;
+  char *mine = s_raw + warp * a.warp_smem;
+  float4 *slots = reinterpret_cast<float4 *>(mine);  // [slots][lane] y
+  const WarpCache<VALS> cache(mine + a.slots * kSlotBytesBsb, a.cache_cap);
+  if (warp == 0) tc::tmem_alloc(&s_tmem, kPersistTmem);
   int my_count = 0;
   const int n_units = s.N * chunks;
-  const int cap = C::kPerWarp < a.cache_cap ? C::kPerWarp : a.cache_cap;
-  for (int u = gw; u < n_units && my_count < cap; u += warps_total, ++my_count) {
-    if (lane == 0) {
-      const int row = u / chunks;
-      const int e0 = a.row_ptr[row], e1 = a.row_ptr[row + 1];
-      Entry &m = mine[my_count];
-      m.row = row;
-      m.chunk = u - row * chunks;
-      m.degpos = uint32_t(e1 - e0) | (uint32_t(KIND == VAL_PM1 ? a.npos[row] : e1 - e0) << 8);
-      for (int q = 0; q < kPersistMaxDeg; ++q) {
-        m.col[q] = q < e1 - e0 ? a.col[e0 + q] : 0;
-        if constexpr (VALS) m.val[q] = q < e1 - e0 ? entry_value<KIND>(a, e0 + q) : 0.f;
+  for (int u = gw; u < n_units && my_count < a.cache_cap; u += warps_total, ++my_count) {
+    const int row = u / chunks;
+    cache.fill(a, my_count, row, u - row * chunks, lane);
+  }
+  tc::tc_fence_before();
+  __syncthreads();
+  tc::tc_fence_after();
+  const uint32_t tm = s_tmem + (uint32_t(warp & 3) << 21) + uint32_t(warp >> 2) * kWarpTmem;
+  const int resident = min(my_count, kTmemItemsBsb + a.slots);
+  auto put = [&](int q, const float (&ys)[4]) {
+    if (q < kTmemItemsBsb) {
+      const uint32_t r[4] = {__float_as_uint(ys[0]), __float_as_uint(ys[1]), __float_as_uint(ys[2]),
+                             __float_as_uint(ys[3])};
+      tc::tmem_st_32x32b_x4(tm + uint32_t(q) * 4u, r);
+    } else {
+      slots[(q - kTmemItemsBsb) * 32 + lane] = make_float4(ys[0], ys[1], ys[2], ys[3]);
+    }
+  };
+  auto get = [&](int q, float (&ys)[4]) {
+    if (q < kTmemItemsBsb) {
+      uint32_t r[4];
+      tc::tmem_ld_32x32b_x4_nowait(tm + uint32_t(q) * 4u, r);
+      tc::tmem_wait_ld();
+      tc::reg_fence_n(r);
+#pragma unroll
+      for (int j = 0; j < 4; ++j) ys[j] = __uint_as_float(r[j]);
+    } else {
+      const float4 v = slots[(q - kTmemItemsBsb) * 32 + lane];
+      ys[0] = v.x; ys[1] = v.y; ys[2] = v.z; ys[3] = v.w;
+    }
+  };
+  auto offset = [&](int q) {
+    const int2 it = cache.item[q];
+    return size_t(it.x) * s.Cp + it.y * kColsPerWarp + lane * 4;
+  };
+  for (int q = 0; q < resident; ++q) {
+    float ys[4];
+    load_row<4>(s.y + offset(q), ys);
+    put(q, ys);
+  }
+  bool ok = true;
+  for (int n = a.n_begin; ok && n < a.n_end; ++n) {
+    const float *Fin = s.fx_of(n);
+    float *Fout = s.fx_of(n + 1);
+    const bool last = n + 1 == a.n_end;
+    const uint32_t tag = tag_of(n, a.n_begin, kTagPos), next = last ? 0u : tag_of(n + 1, a.n_begin, kTagPos);
+    tc::tmem_wait_st();
+    for (int q = 0; q < my_count; ++q) {
+      const int2 it = cache.item[q];
+      const int i = it.x, c4 = it.y * kColsPerWarp + lane * 4;
+      const size_t off = size_t(i) * s.Cp + c4;
+      const bool live = c4 < s.C;
+      float xs[4], ys[4];
+      if (q >= resident) load_row<4>(s.y + off, ys);
+      Pos4 f[kPersistMaxDeg], own;  // own: this lane stored it the step before, or it stood there before this launch
+      {
+        const float *F = Fin + c4;
+        const int4 ca = cache.cols[2 * q], cb = cache.cols[2 * q + 1];
+        uint64_t t0 = 0;
+        for (unsigned it = 0;; ++it) {  // until every live lane's entries are of step n
+          own.load(Fin + off);
+          f[0].load(F + size_t(ca.x) * s.Cp);
+          f[1].load(F + size_t(ca.y) * s.Cp);
+          f[2].load(F + size_t(ca.z) * s.Cp);
+          f[3].load(F + size_t(ca.w) * s.Cp);
+          if (a.degree > 4) {
+            f[4].load(F + size_t(cb.x) * s.Cp);
+            f[5].load(F + size_t(cb.y) * s.Cp);
+          }
+          if (a.degree > 6) {
+            f[6].load(F + size_t(cb.z) * s.Cp);
+            f[7].load(F + size_t(cb.w) * s.Cp);
+          }
+          uint32_t all = ~0u, any = 0u;
+          auto look = [&](const Pos4 &v) {
+            if (tag) all &= v.w[0] & v.w[1] & v.w[2] & v.w[3];
+            else any |= v.w[0] | v.w[1] | v.w[2] | v.w[3];
+          };
+#pragma unroll
+          for (int e = 0; e < 4; ++e) look(f[e]);
+          if (a.degree > 4) {
+            look(f[4]);
+            look(f[5]);
+          }
+          if (a.degree > 6) {
+            look(f[6]);
+            look(f[7]);
+          }
+          const bool stale = tag ? (all & kTagPos) == 0 : (any & kTagPos) != 0;
+          if (!__any_sync(0xffffffffu, live && stale) || n == a.n_begin) break;
+          if (wait_over(it, t0, a.err)) {
+            ok = false;
+            break;
+          }
+        }
+        if (!ok) break;
+      }
+      const uint32_t meta = cache.meta[q];
+      const int deg = int(meta & 0xffffu), npos = (deg + (int(meta) >> 16)) / 2;
+      const float hi = __ldg(a.h + i);
+#pragma unroll
+      for (int j = 0; j < 4; ++j) xs[j] = __uint_as_float(own.w[j] ^ tag);
+      float g[4] = {0.f, 0.f, 0.f, 0.f};
+      auto add = [&](int e) {  // a weight of 0 past the degree
+        float w;
+        if constexpr (VALS) w = reinterpret_cast<const float *>(cache.vals + 2 * q)[e];
+        else w = e < npos ? 1.f : (e < deg ? -1.f : 0.f);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) g[j] = fmaf(w, __uint_as_float(f[e].w[j] ^ tag), g[j]);
+      };
+#pragma unroll
+      for (int e = 0; e < 4; ++e) add(e);
+      if (a.degree > 4) {
+        add(4);
+        add(5);
+      }
+      if (a.degree > 6) {
+        add(6);
+        add(7);
+      }
+      if (q < resident) get(q, ys);
+      sb_advance4_bsb<P>(s, a.t, n, c4, g, hi, xs, ys);
+      if (live) {
+        if (!(n == a.skip_step && blockIdx.x == 0))
+          asm volatile("st.relaxed.gpu.global.v4.u32 [%0], {%1, %2, %3, %4};" ::"l"(Fout + off),
+                       "r"(__float_as_uint(xs[0]) | next), "r"(__float_as_uint(xs[1]) | next),
+                       "r"(__float_as_uint(xs[2]) | next), "r"(__float_as_uint(xs[3]) | next)
+                       : "memory");
+        if (last) store_row<4>(s.x + off, xs);
+      }
+      if (q < resident) {
+        __syncwarp();
+        put(q, ys);
+      } else if (live) {
+        store_row<4>(s.y + off, ys);
       }
     }
   }
-  __syncwarp();
-  unsigned k = 0;
-  for (int n = a.n_begin; n < a.n_end; ++n) {
-    const float *Fin = s.fx_of(n);
-    float *Fout = s.fx_of(n + 1);
-    for (int q = 0; q < my_count; ++q) {
-      const Entry &m = mine[q];
-      const int i = m.row, c4 = m.chunk * kColsPerWarp + lane * 4;
-      const size_t off = size_t(i) * s.Cp + c4;
-      const float4 xv = *reinterpret_cast<const float4 *>(s.x + off);
-      const float4 yv = *reinterpret_cast<const float4 *>(s.y + off);
-      const int deg = int(m.degpos & 0xffu), npos = int(m.degpos >> 8);
-      float4 f[kPersistMaxDeg];
-#pragma unroll
-      for (int e = 0; e < kPersistMaxDeg; ++e)
-        f[e] = e < deg ? __ldcg(reinterpret_cast<const float4 *>(Fin + size_t(m.col[e]) * s.Cp + c4))
-                       : make_float4(0.f, 0.f, 0.f, 0.f);
-      float g[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-      for (int e = 0; e < kPersistMaxDeg; ++e) {
-        float w = 0.f;
-        if (e < deg) {
-          if constexpr (VALS) w = m.val[e];
-          else w = e < npos ? 1.f : -1.f;
-        }
-        g[0] = fmaf(w, f[e].x, g[0]);
-        g[1] = fmaf(w, f[e].y, g[1]);
-        g[2] = fmaf(w, f[e].z, g[2]);
-        g[3] = fmaf(w, f[e].w, g[3]);
-      }
-      sb_update4_bsb<P>(s, a.t, n, i, c4, g, __ldg(a.h + i), xv, yv, Fout);
-    }
-    if (!grid_barrier(a.bar, ++k, a.err, n == a.skip_step && blockIdx.x == 0)) break;
+  tc::tmem_wait_st();
+  for (int q = 0; q < resident; ++q) {
+    float ys[4];
+    get(q, ys);
+    if (cache.item[q].y * kColsPerWarp + lane * 4 < s.C) store_row<4>(s.y + offset(q), ys);
+  }
+  tc::tc_fence_before();
+  __syncthreads();
+  if (warp == 0) {
+    tc::tc_fence_after();
+    tc::tmem_dealloc(s_tmem, kPersistTmem);
   }
 }
 
@@ -351,168 +647,151 @@ static const void *persistent_bsb_fn_k(int P) {
   }
 }
 
+// BF16 values are FP32 in the ELL form
 static const void *persistent_bsb_fn(int P, int kind) {
-  switch (kind) {
-    case VAL_PM1: return persistent_bsb_fn_k<VAL_PM1>(P);
-    case VAL_F32: return persistent_bsb_fn_k<VAL_F32>(P);
-    default: return persistent_bsb_fn_k<VAL_BF16>(P);
-  }
+  return kind == VAL_PM1 ? persistent_bsb_fn_k<VAL_PM1>(P) : persistent_bsb_fn_k<VAL_F32>(P);
 }
 
-// Items mode with 128-column items (W = 4 on a whole warp) runs as W = 8 on
-// half warps (LPI = 16); rows mode and 256-column items keep LPI = 32.
-template <bool ROWS, int KIND, int W>
+template <int KIND, int LPI>
 static const void *persistent_fn_p(int P) {
-  constexpr bool HALF = !ROWS && W == 4;
-  constexpr int WK = HALF ? 8 : W, LPI = HALF ? 16 : 32;
   switch (P) {
-    case 1: return (const void *)k_solve_csr_persistent<1, ROWS, KIND, WK, LPI>;
-    case 2: return (const void *)k_solve_csr_persistent<2, ROWS, KIND, WK, LPI>;
-    case 4: return (const void *)k_solve_csr_persistent<4, ROWS, KIND, WK, LPI>;
-    case 8: return (const void *)k_solve_csr_persistent<8, ROWS, KIND, WK, LPI>;
-    case 16: return (const void *)k_solve_csr_persistent<16, ROWS, KIND, WK, LPI>;
-    case 32: return (const void *)k_solve_csr_persistent<32, ROWS, KIND, WK, LPI>;
-    case 64: return (const void *)k_solve_csr_persistent<64, ROWS, KIND, WK, LPI>;
-    case 128: return (const void *)k_solve_csr_persistent<128, ROWS, KIND, WK, LPI>;
+    case 1: return (const void *)k_solve_csr_persistent<1, KIND, LPI>;
+    case 2: return (const void *)k_solve_csr_persistent<2, KIND, LPI>;
+    case 4: return (const void *)k_solve_csr_persistent<4, KIND, LPI>;
+    case 8: return (const void *)k_solve_csr_persistent<8, KIND, LPI>;
+    case 16: return (const void *)k_solve_csr_persistent<16, KIND, LPI>;
+    case 32: return (const void *)k_solve_csr_persistent<32, KIND, LPI>;
+    case 64: return (const void *)k_solve_csr_persistent<64, KIND, LPI>;
+    case 128: return (const void *)k_solve_csr_persistent<128, KIND, LPI>;
     default: return nullptr;
   }
 }
 
-template <bool ROWS, int W>
-static const void *persistent_fn_k(int P, int kind) {
-  switch (kind) {
-    case VAL_PM1: return persistent_fn_p<ROWS, VAL_PM1, W>(P);
-    case VAL_F32: return persistent_fn_p<ROWS, VAL_F32, W>(P);
-    default: return persistent_fn_p<ROWS, VAL_BF16, W>(P);
-  }
+static const void *persistent_fn(int P, int kind, int lpi) {
+  if (kind == VAL_PM1) return lpi == 32 ? persistent_fn_p<VAL_PM1, 32>(P) : persistent_fn_p<VAL_PM1, 16>(P);
+  return lpi == 32 ? persistent_fn_p<VAL_F32, 32>(P) : persistent_fn_p<VAL_F32, 16>(P);
 }
 
-static const void *persistent_fn(int P, bool rows, int kind, int W) {
-  if (W == 8) return rows ? persistent_fn_k<true, 8>(P, kind) : persistent_fn_k<false, 8>(P, kind);
-  return rows ? persistent_fn_k<true, 4>(P, kind) : persistent_fn_k<false, 4>(P, kind);
-}
+// Items of 256 columns on whole warps when R * P allows it, else of 128 on half warps.
+static int persist_lpi(int Cp) { return Cp % 256 == 0 ? 32 : (Cp % 128 == 0 ? 16 : 0); }
 
-static int per_warp(bool rows, int kind) {
-  const bool vals = kind != VAL_PM1;
-  if (rows) return vals ? Cache<true, true>::kPerWarp : Cache<true, false>::kPerWarp;
-  return vals ? Cache<false, true>::kPerWarp : Cache<false, false>::kPerWarp;
-}
-
-// W = 8 columns per lane when R * P allows it, else 4.
-static int persist_w(int Cp) { return Cp % 256 == 0 ? 8 : (Cp % 128 == 0 ? 4 : 0); }
-
-int persistent_barrier_words() { return int(kBarStride * (kBarGroups + 1)); }
-
-// Test hook: SBQA_TEST_PERSIST_CACHE=k caches at most k items or rows per
-// warp, so that small instances take mode 3 (not for production use).
+// The test hook of solve_streaming.cu that caps a warp's cache; here it sends
+// instances with more items to the streaming form (ballistic: per step).
 static int cache_cap_hook() {
   const char *v = std::getenv("SBQA_TEST_PERSIST_CACHE");
   const int k = v ? std::atoi(v) : 0;
   return k > 0 ? k : (1 << 30);
 }
 
+// Blocks of the grid: one per SM, as the registers and shared memory of every
+// instantiation allow (0 when one does not fit the device, or the streaming
+// form's blocks do not).  Also sets their shared-memory limits, which last for
+// the context.
 int persistent_blocks() {
-  int dev = 0, sms = 0, best = 1 << 30;
+  int dev = 0, sms = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  // the smallest co-resident count over all instantiations, so any of them fits the grid
+  auto fits = [](const void *fn) {
+    int per_sm = 0;
+    return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kPersistSmem) == cudaSuccess &&
+           cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kPersistThreads, kPersistSmem) == cudaSuccess &&
+           per_sm >= 1;
+  };
   const int Ps[8] = {1, 2, 4, 8, 16, 32, 64, 128};
   for (int P : Ps)
-    for (int kind = 0; kind < 3; ++kind)
-      for (int rows = 0; rows < 2; ++rows)
-        for (int W = 4; W <= 8; W += 4) {
-          int per_sm = 0;
-          if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, persistent_fn(P, rows != 0, kind, W), 256,
-                                                            kPersistSmem) != cudaSuccess)
-            return 0;
-          best = per_sm < best ? per_sm : best;
-        }
-  for (int P : Ps)
-    for (int kind = 0; kind < 3; ++kind) {
-      int per_sm = 0;
-      if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, persistent_bsb_fn(P, kind), 256, kPersistSmem) !=
-          cudaSuccess)
+    for (int kind : {VAL_PM1, VAL_F32})
+      if (!fits(persistent_fn(P, kind, 16)) || !fits(persistent_fn(P, kind, 32)) || !fits(persistent_bsb_fn(P, kind)))
         return 0;
-      best = per_sm < best ? per_sm : best;
-    }
-  return sms * best;
+  return streaming_fits() ? sms : 0;
+}
+
+// Lays out a warp's shared memory: its share of `units` items of `eb` bytes,
+// and state slots of `slot` bytes for the passes of `per_pass` items beyond
+// the `tmem` ones, at most kMaxSlots of them.
+static void split_smem(PersistArgs *a, long long units, int warps, int eb, int per_pass, int tmem, int slot) {
+  a->cache_cap = int((units + warps - 1) / warps);
+  const int cache = (a->cache_cap * eb + 15) / 16 * 16;
+  const int passes = (a->cache_cap + per_pass - 1) / per_pass;
+  a->slots = std::max(0, std::min({(kWarpSmem - cache) / slot, passes - tmem, kMaxSlots}));
+  a->warp_smem = cache + a->slots * slot;
+}
+
+// Items of the ballistic form a warp takes at most before the streaming form
+// is the faster one (L = 20, R*P = 2048: 35 items, 70 us per step against 71;
+// L = 24: 61 items, 126 against 119).
+static bool bsb_resident(int N, int Cp, int blocks) {
+  return (long long)N * (Cp / kColsPerWarp) <=
+         (long long)blocks * kPersistWarps * std::min(kMaxPasses, cache_cap_hook());
 }
 
 bool persistent_bsb_ok(int N, int Cp, int max_degree, int kind, int blocks) {
   if (blocks <= 0 || max_degree > kPersistMaxDeg || Cp % kColsPerWarp != 0) return false;
-  return (long long)N * (Cp / kColsPerWarp) <= (long long)blocks * 8 * std::min<long long>(per_warp(false, kind),
-                                                                                         cache_cap_hook());
+  return bsb_resident(N, Cp, blocks) || streaming_bsb_ok(N, Cp, max_degree, kind, blocks * kStreamBlocksPerSm);
+}
+
+static PersistArgs persist_args(const StateView &s, const CsrView &J, const StepTables &t, int n_begin, int n_end,
+                                int *err) {
+  PersistArgs a;
+  a.s = s;
+  a.h = J.h;
+  a.ell_col = J.ell_col;
+  a.ell_meta = J.ell_meta;
+  a.ell_val = J.ell_val;
+  a.t = t;
+  a.n_begin = n_begin;
+  a.n_end = n_end;
+  a.err = err;
+  // test hook for the bounded waits: SBQA_TEST_SKIP_BARRIER_STEP=n makes block 0
+  // keep the codes of step n of a launch that runs it (not for production use)
+  const char *skip = std::getenv("SBQA_TEST_SKIP_BARRIER_STEP");
+  a.skip_step = skip ? std::atoi(skip) : -1;
+  a.degree = J.max_degree;
+  a.cache_cap = a.slots = a.warp_smem = 0;
+  return a;
+}
+
+// `other`: the f buffer of step n_begin + 1, cleared so that none of its
+// generation bits is left from an earlier launch.
+static cudaError_t launch_persist(const void *fn, PersistArgs &a, int kind, void *other, size_t bytes, int blocks,
+                                  cudaStream_t st) {
+  if (!fn || !a.ell_col || !a.ell_meta || (kind != VAL_PM1 && !a.ell_val)) return cudaErrorInvalidValue;
+  const cudaError_t e = cudaMemsetAsync(other, 0, bytes, st);
+  if (e != cudaSuccess) return e;
+  void *args[] = {&a};
+  return cudaLaunchCooperativeKernel(fn, dim3(blocks), dim3(kPersistThreads), args,
+                                     size_t(a.warp_smem) * kPersistWarps, st);
 }
 
 cudaError_t launch_solve_csr_persistent_bsb(const StateView &s, const CsrView &J, const StepTables &t, int n_begin,
                                             int n_end, unsigned *bar, int *err, int blocks, cudaStream_t st) {
-  PersistArgs a;
-  a.s = s;
-  a.row_ptr = J.row_ptr;
-  a.col = J.col;
-  a.npos = J.npos;
-  a.val = J.val;
-  a.h = J.h;
-  a.ell_col = J.ell_col;
-  a.ell_meta = J.ell_meta;
-  a.ell_val = J.ell_val;
-  a.t = t;
-  a.n_begin = n_begin;
-  a.n_end = n_end;
-  a.bar = bar;
-  a.err = err;
-  const char *skip = std::getenv("SBQA_TEST_SKIP_BARRIER_STEP");
-  a.skip_step = skip ? std::atoi(skip) : -1;
-  a.cache_cap = cache_cap_hook();
-  const void *fn = persistent_bsb_fn(s.P, J.kind);
-  if (!fn || !persistent_bsb_ok(s.N, s.Cp, kPersistMaxDeg, J.kind, blocks)) return cudaErrorInvalidValue;
-  cudaError_t e = cudaMemsetAsync(bar, 0, persistent_barrier_words() * sizeof(unsigned), st);
-  if (e != cudaSuccess) return e;
-  void *args[] = {&a};
-  return cudaLaunchCooperativeKernel(fn, dim3(blocks), dim3(256), args, kPersistSmem, st);
+  if (!bsb_resident(s.N, s.Cp, blocks))
+    return launch_solve_csr_streaming_bsb(s, J, t, n_begin, n_end, bar, err, blocks * kStreamBlocksPerSm, st);
+  PersistArgs a = persist_args(s, J, t, n_begin, n_end, err);
+  split_smem(&a, (long long)s.N * (s.Cp / kColsPerWarp), blocks * kPersistWarps, entry_bytes(J.kind != VAL_PM1), 1,
+             kTmemItemsBsb, kSlotBytesBsb);
+  return launch_persist(persistent_bsb_fn(s.P, J.kind), a, J.kind, s.fx_of(n_begin + 1),
+                        size_t(s.N) * s.Cp * sizeof(float), blocks, st);
 }
 
-
 int persistent_mode(int N, int Cp, int max_degree, int kind, int blocks, bool force_rows, bool ell) {
-  const int W = persist_w(Cp);
-  if (blocks <= 0 || max_degree > kPersistMaxDeg || W == 0) return 0;
-  const long long warps = (long long)blocks * 8, cap = cache_cap_hook();
-  if (!force_rows && (long long)N * (Cp / (32 * W)) <= warps * std::min<long long>(per_warp(false, kind), cap)) return 1;
-  if ((long long)N <= warps * std::min<long long>(per_warp(true, kind), cap)) return 2;
-  if (!force_rows && ell) return 3;
-  return 0;
+  const int lpi = persist_lpi(Cp);
+  if (blocks <= 0 || max_degree > kPersistMaxDeg || lpi == 0 || !ell) return 0;
+  const long long items = (long long)N * (Cp / (8 * lpi)), warps = (long long)blocks * kPersistWarps;
+  const long long most = std::min<long long>(kMaxPasses * (32 / lpi), cache_cap_hook());
+  if (!force_rows && items <= warps * most) return kPersistResident;
+  return streaming_mode(N, Cp, max_degree, kind, blocks * kStreamBlocksPerSm, force_rows, ell);
 }
 
 cudaError_t launch_solve_csr_persistent(const StateView &s, const CsrView &J, const StepTables &t, int n_begin,
                                         int n_end, unsigned *bar, int *err, int blocks, int mode, cudaStream_t st) {
-  PersistArgs a;
-  a.s = s;
-  a.row_ptr = J.row_ptr;
-  a.col = J.col;
-  a.npos = J.npos;
-  a.val = J.val;
-  a.h = J.h;
-  a.ell_col = J.ell_col;
-  a.ell_meta = J.ell_meta;
-  a.ell_val = J.ell_val;
-  a.t = t;
-  a.n_begin = n_begin;
-  a.n_end = n_end;
-  a.bar = bar;
-  a.err = err;
-  // test hook for the barrier timeout: SBQA_TEST_SKIP_BARRIER_STEP=n makes block 0
-  // skip its arrival after step n of a launch that runs it (not for production use)
-  const char *skip = std::getenv("SBQA_TEST_SKIP_BARRIER_STEP");
-  a.skip_step = skip ? std::atoi(skip) : -1;
-  a.cache_cap = cache_cap_hook();
-  void *args[] = {&a};
-  const int W = persist_w(s.Cp);
-  const void *fn = (mode == 1 || mode == 2 || mode == 3) && W ? persistent_fn(s.P, mode == 2, J.kind, W) : nullptr;
-  if (!fn || (mode == 3 && (!J.ell_col || !J.ell_meta || (J.kind != VAL_PM1 && !J.ell_val))))
-    return cudaErrorInvalidValue;
-  cudaError_t e = cudaMemsetAsync(bar, 0, persistent_barrier_words() * sizeof(unsigned), st);
-  if (e != cudaSuccess) return e;
-  return cudaLaunchCooperativeKernel(fn, dim3(blocks), dim3(256), args, kPersistSmem, st);
+  const int lpi = persist_lpi(s.Cp);
+  if (mode != kPersistResident)
+    return launch_solve_csr_streaming(s, J, t, n_begin, n_end, bar, err, blocks * kStreamBlocksPerSm, mode, st);
+  PersistArgs a = persist_args(s, J, t, n_begin, n_end, err);
+  split_smem(&a, (long long)s.N * (s.Cp / (8 * lpi)), blocks * kPersistWarps, entry_bytes(J.kind != VAL_PM1), 32 / lpi,
+             kTmemPasses, kSlotBytes);
+  return launch_persist(persistent_fn(s.P, J.kind, lpi), a, J.kind, s.f_of(n_begin + 1), size_t(s.N) * s.Cp, blocks,
+                        st);
 }
 
 }  // namespace sbqa

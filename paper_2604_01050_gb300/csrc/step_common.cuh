@@ -255,46 +255,40 @@ __device__ __forceinline__ void sb_update4c(const StateView &s, const LaneConsts
   *reinterpret_cast<uint32_t *>(Fout + off) = code;
 }
 
+// dt * J_perp of the runs of W consecutive columns (one load per run in the
+// lane; c0 is the first column, and a column past C reads nothing).
+template <int P, int W>
+__device__ __forceinline__ void load_kj(const float *kjn, int C, int c0, float (&kj)[P >= W ? 1 : W / P]) {
+#pragma unroll
+  for (int r = 0; r < (P >= W ? 1 : W / P); ++r) kj[r] = (c0 + r * P < C) ? __ldg(kjn + c0 / P + r) : 0.f;
+}
+
 // Generalisation of sb_update4c to W consecutive columns per lane (W = 4,
-// 8 or 16; W >= P or P divides W).  Ring neighbours inside the lane's
-// columns are registers; across lanes (P > W) they come by shuffle from the
-// neighbouring lane of the same run.  Same arithmetic as sb_update4.
-template <int P, int W, bool GEN = true>
-__device__ __forceinline__ void sb_updateW(const StateView &s, const StepTables &t, float ka, float dnext, int n,
-                                           int i, int c0, const float (&G)[W], float hi, float (&xs)[W],
-                                           float (&ys)[W], uint8_t *Fout) {
-  float xm[W], xp[W];
-  ring_nb<P, W, GEN>(xs, s.Pr, xm, xp);  // all lanes take part (shuffles)
-  if (c0 >= s.C) return;
-  const float *kjn = t.kj + size_t(n) * t.R;
-  const float2 kc2 = make_float2(t.kc, t.kc), mka2 = make_float2(-ka, -ka), kx2 = make_float2(t.kx, t.kx);
-  const float2 h2 = make_float2(hi, hi);
-  uint32_t code[W / 4];
+// 8 or 16; W >= P or P divides W), in registers: xs, ys become the next
+// state and code the next f codes; columns past C keep their state and get
+// the code of f = 0.  xm, xp: the ring neighbours (ring_nb).  Same arithmetic
+// as sb_update4.  A lane is ragged only when P < W: with P >= W its columns
+// lie on one side of C.
+template <int P, int W>
+__device__ __forceinline__ void sb_advanceW(int C, float kc, float kx, float ka, float dnext,
+                                            const float (&kj)[P >= W ? 1 : W / P], int c0, const float (&G)[W],
+                                            float hi, const float (&xm)[W], const float (&xp)[W], float (&xs)[W],
+                                            float (&ys)[W], uint32_t (&code)[W / 4]) {
 #pragma unroll
   for (int q = 0; q < W / 4; ++q) code[q] = 0;
-  // dt * J_perp of the run of each column (one load per run in the lane)
-  float kjv[W];
-  if constexpr (P >= W) {
-    const float k = (c0 < s.C) ? __ldg(kjn + c0 / P) : 0.f;
-#pragma unroll
-    for (int j = 0; j < W; ++j) kjv[j] = k;
-  } else {
-#pragma unroll
-    for (int r = 0; r < W / P; ++r) {
-      const float k = (c0 + r * P < s.C) ? __ldg(kjn + c0 / P + r) : 0.f;
-#pragma unroll
-      for (int u = 0; u < P; ++u) kjv[r * P + u] = k;
-    }
-  }
+  if (c0 >= C) return;
+  const float2 kc2 = make_float2(kc, kc), mka2 = make_float2(-ka, -ka), kx2 = make_float2(kx, kx);
+  const float2 h2 = make_float2(hi, hi);
 #pragma unroll
   for (int pr = 0; pr < W / 2; ++pr) {
     const int a = 2 * pr, b = a + 1;
-    const float kja = kjv[a], kjb = kjv[b];
+    const float kja = kj[P >= W ? 0 : a / P], kjb = kj[P >= W ? 0 : b / P];
     const float2 x2 = make_float2(xs[a], xs[b]);
     float2 y2 = make_float2(ys[a], ys[b]);
     y2 = __ffma2_rn(kc2, __fadd2_rn(make_float2(G[a], G[b]), h2), y2);
     y2 = __ffma2_rn(mka2, x2, y2);
-    y2 = __ffma2_rn(make_float2(kja, kjb), __fadd2_rn(make_float2(xm[a], xm[b]), make_float2(xp[a], xp[b])), y2);
+    // scalar adds: the neighbours of a column pair straddle register pairs
+    y2 = __ffma2_rn(make_float2(kja, kjb), make_float2(__fadd_rn(xm[a], xp[a]), __fadd_rn(xm[b], xp[b])), y2);
     const float2 xn2 = __ffma2_rn(kx2, y2, x2);
     const float xo[2] = {xn2.x, xn2.y}, yo[2] = {y2.x, y2.y};
 #pragma unroll
@@ -302,29 +296,62 @@ __device__ __forceinline__ void sb_updateW(const StateView &s, const StepTables 
       const int j = a + u;
       const float xc = fminf(fmaxf(xo[u], -1.f), 1.f);  // wall
       const float yn = (xc != xo[u]) ? 0.f : yo[u];
-      uint32_t cj = 1u + uint32_t(xc > dnext) - uint32_t(xc < -dnext);
-      if (c0 + j >= s.C) {  // ragged tail (P < 4): padding column untouched
-        cj = kFZero;
+      if (P < W && c0 + j >= C) {  // ragged tail: padding column untouched
+        code[j / 4] += uint32_t(kFZero) << (8 * (j % 4));
       } else {
         xs[j] = xc;
         ys[j] = yn;
+        // code f + 1 counts the two thresholds x has passed
+        if (xc >= -dnext) code[j / 4] += 1u << (8 * (j % 4));
+        if (xc > dnext) code[j / 4] += 1u << (8 * (j % 4));
       }
-      code[j / 4] |= cj << (8 * (j % 4));
     }
   }
-  const size_t off = size_t(i) * s.Cp + c0;
+}
+
+template <int W>
+__device__ __forceinline__ void store_codes(uint8_t *p, const uint32_t (&code)[W / 4]) {
+  if constexpr (W == 4) {
+    *reinterpret_cast<uint32_t *>(p) = code[0];
+  } else if constexpr (W == 8) {
+    *reinterpret_cast<uint2 *>(p) = make_uint2(code[0], code[1]);
+  } else {
+    *reinterpret_cast<uint4 *>(p) = make_uint4(code[0], code[1], code[2], code[3]);
+  }
+}
+
+// W consecutive columns of one row to and from memory.
+template <int W>
+__device__ __forceinline__ void load_row(const float *p, float (&v)[W]) {
 #pragma unroll
   for (int q = 0; q < W / 4; ++q) {
-    *reinterpret_cast<float4 *>(s.x + off + 4 * q) = make_float4(xs[4 * q], xs[4 * q + 1], xs[4 * q + 2], xs[4 * q + 3]);
-    *reinterpret_cast<float4 *>(s.y + off + 4 * q) = make_float4(ys[4 * q], ys[4 * q + 1], ys[4 * q + 2], ys[4 * q + 3]);
+    const float4 a = *reinterpret_cast<const float4 *>(p + 4 * q);
+    v[4 * q] = a.x; v[4 * q + 1] = a.y; v[4 * q + 2] = a.z; v[4 * q + 3] = a.w;
   }
-  if constexpr (W == 4) {
-    *reinterpret_cast<uint32_t *>(Fout + off) = code[0];
-  } else if constexpr (W == 8) {
-    *reinterpret_cast<uint2 *>(Fout + off) = make_uint2(code[0], code[1]);
-  } else {
-    *reinterpret_cast<uint4 *>(Fout + off) = make_uint4(code[0], code[1], code[2], code[3]);
-  }
+}
+template <int W>
+__device__ __forceinline__ void store_row(float *p, const float (&v)[W]) {
+#pragma unroll
+  for (int q = 0; q < W / 4; ++q)
+    *reinterpret_cast<float4 *>(p + 4 * q) = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+}
+
+// sb_advanceW with the state and the codes written back to global memory.
+template <int P, int W, bool GEN = true>
+__device__ __forceinline__ void sb_updateW(const StateView &s, const StepTables &t, float ka, float dnext, int n,
+                                           int i, int c0, const float (&G)[W], float hi, float (&xs)[W],
+                                           float (&ys)[W], uint8_t *Fout) {
+  float xm[W], xp[W];
+  ring_nb<P, W, GEN>(xs, s.Pr, xm, xp);  // all lanes take part (shuffles)
+  if (c0 >= s.C) return;
+  float kj[P >= W ? 1 : W / P];
+  load_kj<P, W>(t.kj + size_t(n) * t.R, s.C, c0, kj);
+  uint32_t code[W / 4];
+  sb_advanceW<P, W>(s.C, t.kc, t.kx, ka, dnext, kj, c0, G, hi, xm, xp, xs, ys, code);
+  const size_t off = size_t(i) * s.Cp + c0;
+  store_row<W>(s.x + off, xs);
+  store_row<W>(s.y + off, ys);
+  store_codes<W>(Fout + off, code);
 }
 
 // Value of f encoded in byte q of a packed word of f codes.
@@ -338,10 +365,11 @@ __device__ __forceinline__ float fdec(uint32_t w, int q) {
 // -(2^23 + 1) gives f = code - 1 in {-1, 0, 1} exactly, and each lane of
 // __ffma2_rn is the ordinary round-to-nearest fma: the sums equal
 // fmaf(w, fdec(...), g) term by term, in the same order.
+// Codes that carry a bit above the value take another offset.
 template <int W>
-__device__ __forceinline__ void acc_codes(float (&g)[W], float w, const uint32_t *cw) {
+__device__ __forceinline__ void acc_codes_off(float (&g)[W], float w, const uint32_t *cw, float offset) {
   const float2 w2 = make_float2(w, w);
-  const float2 off = make_float2(-8388609.f, -8388609.f);
+  const float2 off = make_float2(offset, offset);
 #pragma unroll
   for (int q = 0; q < W / 4; ++q) {
 #pragma unroll
@@ -357,14 +385,16 @@ __device__ __forceinline__ void acc_codes(float (&g)[W], float w, const uint32_t
   }
 }
 
-// sb_update4 with f(x) = x: same momentum, position and wall arithmetic,
-// writes the new x into the f buffer of the next step.
+template <int W>
+__device__ __forceinline__ void acc_codes(float (&g)[W], float w, const uint32_t *cw) {
+  acc_codes_off<W>(g, w, cw, -8388609.f);
+}
+
+// sb_update4 with f(x) = x, in registers: same momentum, position and wall
+// arithmetic; xs, ys become the next state (columns past C keep theirs).
 template <int P>
-__device__ __forceinline__ void sb_update4_bsb(const StateView &s, const StepTables &t, int n, int i, int c4,
-                                               const float G[4], float hi, float4 xv, float4 yv, float *Fout) {
-  const size_t off = size_t(i) * s.Cp + c4;
-  float xs[4] = {xv.x, xv.y, xv.z, xv.w};
-  float ys[4] = {yv.x, yv.y, yv.z, yv.w};
+__device__ __forceinline__ void sb_advance4_bsb(const StateView &s, const StepTables &t, int n, int c4,
+                                                const float (&G)[4], float hi, float (&xs)[4], float (&ys)[4]) {
   float xm[4], xp[4];
   ring_neighbours<P>(xs, s.Pr, xm, xp);  // all lanes take part (shuffles)
   if (c4 >= s.C) return;                 // padding columns past R * P
@@ -380,7 +410,6 @@ __device__ __forceinline__ void sb_update4_bsb(const StateView &s, const StepTab
   }
   const float2 kc2 = make_float2(t.kc, t.kc), mka2 = make_float2(-ka, -ka);
   const float2 kx2 = make_float2(t.kx, t.kx), h2 = make_float2(hi, hi);
-  float xo[4], yo[4];
 #pragma unroll
   for (int q = 0; q < 2; ++q) {
     const int a = 2 * q, b = 2 * q + 1;
@@ -390,25 +419,31 @@ __device__ __forceinline__ void sb_update4_bsb(const StateView &s, const StepTab
     y2 = __ffma2_rn(mka2, x2, y2);
     y2 = __ffma2_rn(make_float2(kj[a], kj[b]), __fadd2_rn(make_float2(xm[a], xm[b]), make_float2(xp[a], xp[b])), y2);
     const float2 xn2 = __ffma2_rn(kx2, y2, x2);
-    xo[a] = xn2.x; xo[b] = xn2.y;
-    yo[a] = y2.x; yo[b] = y2.y;
-  }
+    const float xo[2] = {xn2.x, xn2.y}, yo[2] = {y2.x, y2.y};
 #pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    const float xc = fminf(fmaxf(xo[j], -1.f), 1.f);  // wall: clamping changes x iff |x| > 1
-    float yn = (xc != xo[j]) ? 0.f : yo[j];
-    float xn = xc;
-    if (P < 4 && c4 + j >= s.C) {  // ragged tail: leave the padding column alone
-      xn = xs[j];
-      yn = ys[j];
+    for (int u = 0; u < 2; ++u) {
+      const int j = a + u;
+      if (P < 4 && c4 + j >= s.C) continue;  // ragged tail: leave the padding column alone
+      const float xc = fminf(fmaxf(xo[u], -1.f), 1.f);  // wall: clamping changes x iff |x| > 1
+      ys[j] = (xc != xo[u]) ? 0.f : yo[u];
+      xs[j] = xc;
     }
-    xo[j] = xn;
-    yo[j] = yn;
   }
-  const float4 xnew = make_float4(xo[0], xo[1], xo[2], xo[3]);
-  *reinterpret_cast<float4 *>(s.x + off) = xnew;
-  *reinterpret_cast<float4 *>(s.y + off) = make_float4(yo[0], yo[1], yo[2], yo[3]);
-  *reinterpret_cast<float4 *>(Fout + off) = xnew;
+}
+
+// The same with the state from and to global memory; the new x also goes to
+// the f buffer of the next step.
+template <int P>
+__device__ __forceinline__ void sb_update4_bsb(const StateView &s, const StepTables &t, int n, int i, int c4,
+                                               const float (&G)[4], float hi, float4 xv, float4 yv, float *Fout) {
+  const size_t off = size_t(i) * s.Cp + c4;
+  float xs[4] = {xv.x, xv.y, xv.z, xv.w};
+  float ys[4] = {yv.x, yv.y, yv.z, yv.w};
+  sb_advance4_bsb<P>(s, t, n, c4, G, hi, xs, ys);
+  if (c4 >= s.C) return;
+  store_row<4>(s.x + off, xs);
+  store_row<4>(s.y + off, ys);
+  store_row<4>(Fout + off, xs);
 }
 
 }  // namespace sbqa
