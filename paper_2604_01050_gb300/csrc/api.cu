@@ -227,6 +227,8 @@ sbqa_problem::~sbqa_problem() {
   if (cap_stream) cudaStreamDestroy(cap_stream);
   if (tc_plan) tc_plan_free(tc_plan);
   if (tc4_plan) tc4_plan_free(tc4_plan);
+  if (fx_plan) fx_plan_free(fx_plan);
+  d_fx_digits.release(true); d_fx_h.release(true);
   d_J8.release(true); d_FT.release(true); d_err.release(true);
   d_row_ptr.release(true); d_col.release(true); d_col_pm1.release(true); d_npos.release(true); d_val_f32.release(true);
   d_val_bf16.release(true); d_dense_f32.release(true); d_h.release(true); d_e_i32.release(true);
@@ -641,6 +643,27 @@ int prepare_tc_values(sbqa_problem *p) {
   return SBQA_OK;
 }
 
+// The fixed-point readout operands of a real J, from its FP64 copy on the
+// device.  Without the memory for them (or with row sums past the FP64 range)
+// the FP64 readout on the CUDA cores serves.
+int prepare_fx(sbqa_problem *p) {
+  if (p->fx_tried || !fx_eligible(p->Kp)) return SBQA_OK;
+  p->fx_tried = true;
+  DevBuf<unsigned long long> scratch;
+  if (p->d_fx_digits.alloc(fx_digit_bytes(p->Kp)) != cudaSuccess || p->d_fx_h.alloc(p->n) != cudaSuccess ||
+      scratch.alloc(1) != cudaSuccess) {
+    cudaGetLastError();
+    p->d_fx_digits.release();
+    p->d_fx_h.release();
+    return SBQA_OK;
+  }
+  const cudaError_t e = fx_plan_make(&p->fx_plan, p->d_e_f64.p, p->d_h_f64.p, p->n, p->Kp, p->d_fx_digits.p,
+                                     p->d_fx_h.p, scratch.p, nullptr);
+  scratch.release(true);
+  SBQA_CUDA(e);
+  return SBQA_OK;
+}
+
 int prepare_dense_values(sbqa_problem *p, int precision) {
   if (precision == SBQA_PREC_EXACT && (!p->j_integer || p->max_abs_j > kExactMaxAbsJ))
     return fail(SBQA_ERR_UNSUPPORTED, "EXACT precision needs integer J with |J_ij| <= 256");
@@ -669,10 +692,13 @@ int prepare_dense_values(sbqa_problem *p, int precision) {
     }
     p->tc_op = op;
     // the readout runs on the tensor cores too when its energies are integers
-    // and the product is e4m3; otherwise on the CUDA cores (exact int64 or FP64)
-    const int rc = prepare_tc_values(p);
+    // and the product is e4m3, and in fixed point when they are real and the
+    // operands bfloat16; otherwise on the CUDA cores (exact int64 or FP64)
+    int rc = prepare_tc_values(p);
     if (rc != SBQA_OK || (p->is_integer && op == kTcOpF8)) return rc;
-    return upload_readout_values(p);
+    rc = upload_readout_values(p);
+    if (rc != SBQA_OK || p->is_integer || op == kTcOpF8) return rc;
+    return prepare_fx(p);
   }
   {
     const int rc = upload_readout_values(p);
@@ -1270,13 +1296,19 @@ int autotune_tc(sbqa_problem *p) {
 
 cudaError_t issue_readout(sbqa_problem *p, int step, cudaStream_t st) {
   const StateView s = p->state();
-  // integer dense instances (J and h) on the tensor cores: the sign codes take
-  // the FT buffer of step `step`, which the next step does not read
-  cudaError_t e = p->dense ? (p->use_tc && p->tc_plan && p->is_integer && p->tc_op == kTcOpF8 ? launch_energy_dense_tc(p->tc_plan, s, p->Kp, p->d_FT.p,
-                                                                               step & 1, p->d_err.p, p->energy(),
-                                                                               p->best(), st)
-                                                      : launch_energy_dense(s, p->energy(), p->best(), st))
-                           : launch_energy_csr(s, p->csr_readout(), p->energy(), p->best(), st);
+  // dense instances on the tensor cores: the sign codes take the FT buffer of
+  // step `step`, which the next step does not read
+  const bool tc = p->use_tc && p->tc_plan;
+  const EnergyView E = p->energy();
+  cudaError_t e;
+  if (!p->dense)
+    e = launch_energy_csr(s, p->csr_readout(), E, p->best(), st);
+  else if (tc && p->is_integer && p->tc_op == kTcOpF8)
+    e = launch_energy_dense_tc(p->tc_plan, s, p->Kp, p->d_FT.p, step & 1, p->d_err.p, E, p->best(), st);
+  else if (tc && E.fx)
+    e = launch_energy_dense_fx(p->tc_plan, s, p->Kp, p->d_FT.p, step & 1, p->d_err.p, E, p->best(), st);
+  else
+    e = launch_energy_dense(s, E, p->best(), st);
   if (e != cudaSuccess) return e;
   return launch_best(s, p->energy(), p->best(), step, st);
 }

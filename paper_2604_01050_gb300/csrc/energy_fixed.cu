@@ -1,0 +1,303 @@
+// energy_fixed.cu -- readout energies of real dense instances on the tensor
+// cores, in fixed point.
+//
+// E_c = -(1/2) sum_i s_ic (t_ic + 2 h_i), t_ic = sum_j J_ij s_jc (Sec. II A,
+// Eq. 4 sign; Sec. II B).  An FP64 sum of N^2 Cp terms on the CUDA cores is
+// bound by this chip's FP64 rate (two FMAs per SM and clock): 10.7 ms at
+// N = 2000, R*P = 1024, as long as 700 steps of the solver.  Here J and h are
+// integers X = rint(2^k J), H = rint(2^k h) of 63 bits, with k such that no
+// |t_i + 2 h_i| reaches 2^63, and a bfloat16 operand per byte of X (0 .. 255,
+// exact; the top byte signed): the tensor cores form the eight exact integer
+// sums of a tile (below 2^24 in FP32), which the epilogue joins as
+// acc = 256 acc + digit in 64-bit integers.  Rows and then row blocks add as
+// integers too (the 64-bit values in two 32-bit halves), so the only roundings
+// are those of X and H and one of the result: an energy is closer to the
+// instance's than the FP64 sum in any order, whatever the order.
+// At N = 2000, R*P = 1024 the eight GEMMs (66 GFLOP, operands 64 MB, in L2)
+// and the kernels around them take 0.2 ms instead of 10.7.
+#include <cmath>
+#include <cstdint>
+
+#include "dense_tc_common.cuh"
+
+namespace sbqa {
+
+constexpr int kFxDigits = 8;
+constexpr int kFxMaxKp = 16384;  // 4.3 GB of digits; larger instances keep the FP64 readout
+
+struct FxPlan {
+  CUtensorMap A;  // digits [8 Kp][Kp] bfloat16, most significant plane first
+  const int64_t *H;
+  int k;
+};
+
+// Largest row sum of |J_ij| + 2 |h_i| (bits of a non-negative double, which
+// order as integers do).
+__global__ void __launch_bounds__(256) k_fx_rowsum(const double *J, const double *h, int N, unsigned long long *most) {
+  __shared__ double sm[8];
+  const int i = blockIdx.x;
+  double acc = 0.0;
+  for (int j = threadIdx.x; j < N; j += 256) acc += fabs(J[size_t(i) * N + j]);
+  for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
+  if ((threadIdx.x & 31) == 0) sm[threadIdx.x >> 5] = acc;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < 8; ++w) acc += sm[w];
+    acc += 2.0 * fabs(h[i]);
+    atomicMax(most, static_cast<unsigned long long>(__double_as_longlong(acc)));
+  }
+}
+
+// Bytes of X [N][N] into the planes [8][Kp][Kp], zero padded; H.
+__global__ void k_fx_digits(const double *J, const double *h, int N, int Kp, int k, uint16_t *out, int64_t *H) {
+  const size_t e = size_t(blockIdx.x) * blockDim.x + threadIdx.x;
+  if (e >= size_t(Kp) * Kp) return;
+  const int i = int(e / Kp), j = int(e % Kp);
+  const long long X = (i < N && j < N) ? __double2ll_rn(scalbn(J[size_t(i) * N + j], k)) : 0ll;
+#pragma unroll
+  for (int d = 0; d < kFxDigits; ++d) {
+    const int byte = int((X >> (8 * (kFxDigits - 1 - d))) & 0xff);
+    const float v = d == 0 ? float(int(int8_t(byte))) : float(byte);
+    out[size_t(d) * Kp * Kp + e] = uint16_t(__float_as_uint(v) >> 16);  // at most 8 significant bits: exact
+  }
+  if (j == 0 && i < N) H[i] = __double2ll_rn(scalbn(h[i], k));
+}
+
+// Spins S [N][Cp] (+1, -1; 0 past C) -> bfloat16 [Cp][Kp] in FT buffer b (zeros
+// for padded spins), through 64 x 64 tiles so that both sides are coalesced.
+__global__ void __launch_bounds__(256) k_sign_to_ft16(StateView s, uint16_t *FT, int Kp, int b) {
+  __shared__ int8_t t[64][68];
+  const int i0 = blockIdx.x * 64, c0 = blockIdx.y * 64;
+  for (int q = threadIdx.x; q < 64 * 16; q += 256) {
+    const int r = q >> 4, w = q & 15;
+    uint32_t v = 0;
+    if (i0 + r < s.N) v = *reinterpret_cast<const uint32_t *>(s.Sg + size_t(i0 + r) * s.Cp + c0 + 4 * w);
+    *reinterpret_cast<uint32_t *>(&t[r][4 * w]) = v;
+  }
+  __syncthreads();
+  for (int q = threadIdx.x; q < 64 * 32; q += 256) {
+    const int c = q >> 5, r = (q & 31) * 2;
+    auto code = [](int8_t v) { return v == 0 ? 0u : (v > 0 ? 0x3F80u : 0xBF80u); };
+    const uint32_t v = code(t[r][c]) | (code(t[r + 1][c]) << 16);
+    *reinterpret_cast<uint32_t *>(FT + (size_t(b) * s.Cp + c0 + c) * Kp + i0 + r) = v;
+  }
+}
+
+// One 128 x 128 tile (spin rows x columns) per block: warps 0-15 the epilogue,
+// warp 16 the TMA producer, warp 17 the MMAs.  The K loop runs once per digit,
+// most significant first, into one of two TMEM accumulators, while the
+// epilogue takes in the digit before from the other.  Six stages of 32 KB.
+constexpr int kFxStages = 6, kFxThreads = 18 * 32;
+constexpr int kFxSmem = kFxStages * 2 * kTcTile + 4 * kTcBN * 16 + 1024 + 256;
+static_assert(16 * 32 * 33 * 8 <= kFxStages * 2 * kTcTile, "row reductions must fit the operand stages");
+static_assert(kFxSmem <= 227 * 1024, "shared memory of one block");
+
+__global__ void __launch_bounds__(kFxThreads, 1)
+    k_energy_dense_fx(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB, StateView s,
+                      int Kp, int b, int *err, const int64_t *H, int64_t *part) {
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  uint8_t *sA = smem, *sB = smem + kFxStages * kTcTile;
+  int64_t *cols = reinterpret_cast<int64_t *>(smem + kFxStages * 2 * kTcTile);  // [4 quarters][128 columns][hi, lo]
+  uint64_t *full = reinterpret_cast<uint64_t *>(cols + 4 * kTcBN * 2);
+  uint64_t *empty = full + kFxStages;
+  uint64_t *acc_full = empty + kFxStages, *acc_free = acc_full + 2;
+  uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(acc_free + 2);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int m0 = blockIdx.y * kTcBM, n0 = blockIdx.x * kTcBN;
+  const int KB = Kp / 64, total = KB * kFxDigits;
+  if (threadIdx.x == 0) {
+    for (int q = 0; q < kFxStages; ++q) {
+      tc::mbar_init(&full[q], 1);
+      tc::mbar_init(&empty[q], 1);
+    }
+    for (int q = 0; q < 2; ++q) {
+      tc::mbar_init(&acc_full[q], 1);
+      tc::mbar_init(&acc_free[q], 16);
+    }
+    tc::fence_mbar_init();
+    tc::prefetch_tmap(&mapA);
+    tc::prefetch_tmap(&mapB);
+  }
+  if (warp == 0) tc::tmem_alloc(tmem_slot, 256);
+  tc::tc_fence_before();
+  __syncthreads();
+  tc::tc_fence_after();
+  const uint32_t tmem = *tmem_slot;
+  uint64_t acc[32];
+  if (warp == 16) {
+    if (lane == 0)
+      for (int g = 0; g < total; ++g) {
+        const int st = g % kFxStages, use = g / kFxStages, d = g / KB, kb = g % KB;
+        if (use > 0 && !tc::mbar_wait(&empty[st], (use - 1) & 1, err, tc::ERR_WAIT_EMPTY)) break;
+        tc::mbar_arrive_expect_tx(&full[st], 2 * kTcTile);
+        tc::tma_load_2d(sA + st * kTcTile, &mapA, &full[st], kb * 64, d * Kp + m0);
+        tc::tma_load_2d(sB + st * kTcTile, &mapB, &full[st], kb * 64, b * s.Cp + n0);
+      }
+  } else if (warp == 17) {
+    if (lane == 0) {
+      constexpr uint32_t idesc = tc::idesc_bf16(kTcBM, kTcBN);
+      bool ok = true;
+      for (int d = 0; d < kFxDigits && ok; ++d) {
+        if (d >= 2) ok = tc::mbar_wait(&acc_free[d & 1], (d / 2 - 1) & 1, err, tc::ERR_WAIT_DONE);
+        tc::tc_fence_after();
+        for (int kb = 0; kb < KB && ok; ++kb) {
+          const int g = d * KB + kb, st = g % kFxStages;
+          ok = tc::mbar_wait(&full[st], (g / kFxStages) & 1, err, tc::ERR_WAIT_FULL);
+          if (!ok) break;
+          tc::tc_fence_after();
+          const uint32_t a0 = tc::smem_u32(sA + st * kTcTile), b0 = tc::smem_u32(sB + st * kTcTile);
+#pragma unroll
+          for (int kk = 0; kk < 4; ++kk)
+            tc::mma_bf16(tmem + uint32_t(128 * (d & 1)), tc::smem_desc_sw128(a0 + kk * 32),
+                         tc::smem_desc_sw128(b0 + kk * 32), idesc, (kb | kk) != 0 ? 1u : 0u);
+          tc::mma_commit(&empty[st]);
+        }
+        if (ok) tc::mma_commit(&acc_full[d & 1]);
+      }
+    }
+  } else {
+    const uint32_t at = tmem + (uint32_t((warp & 3) * 32) << 16) + uint32_t(32 * (warp >> 2));
+#pragma unroll
+    for (int j = 0; j < 32; ++j) acc[j] = 0;
+    for (int d = 0; d < kFxDigits; ++d) {
+      if (!tc::mbar_wait(&acc_full[d & 1], (d / 2) & 1, err, tc::ERR_WAIT_DONE)) break;
+      tc::tc_fence_after();
+      __syncwarp();
+      uint32_t g[32];
+      tc::tmem_ld_32x32b_x32(at + uint32_t(128 * (d & 1)), g);
+      tc::reg_fence(g);
+      tc::tc_fence_before();
+      __syncwarp();
+      if (lane == 0) tc::mbar_arrive(&acc_free[d & 1]);
+#pragma unroll
+      for (int j = 0; j < 32; ++j)
+        acc[j] = (acc[j] << 8) + uint64_t(int64_t(__float2int_rn(__uint_as_float(g[j]))));
+    }
+  }
+  // every MMA that read the stages has completed once the last digit is in (or the run has failed):
+  // row reductions reuse them
+  __syncthreads();
+  if (warp < 16) {
+    const int quarter = warp & 3, chunk = warp >> 2;
+    const int i = m0 + quarter * 32 + lane, c0 = n0 + 32 * chunk;
+    int64_t *red = reinterpret_cast<int64_t *>(smem) + size_t(warp) * 32 * 33;
+    uint32_t w[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+    uint64_t h2 = 0;
+    if (i < s.N) {
+      const uint4 *ps = reinterpret_cast<const uint4 *>(s.Sg + size_t(i) * s.Cp + c0);
+      const uint4 u0 = ps[0], u1 = ps[1];
+      w[0] = u0.x; w[1] = u0.y; w[2] = u0.z; w[3] = u0.w; w[4] = u1.x; w[5] = u1.y; w[6] = u1.z; w[7] = u1.w;
+      h2 = 2 * uint64_t(H[i]);
+    }
+#pragma unroll
+    for (int j = 0; j < 32; ++j) {
+      const int8_t si = int8_t(w[j >> 2] >> (8 * (j & 3)));
+      const uint64_t v = acc[j] + h2;
+      red[lane * 33 + j] = int64_t(si == 0 ? 0 : (si > 0 ? v : 0 - v));
+    }
+    __syncwarp();
+    int64_t hi = 0, lo = 0;  // the rows of this quarter in 32-bit halves: no sum can wrap
+#pragma unroll 8
+    for (int r = 0; r < 32; ++r) {
+      const int64_t v = red[r * 33 + lane];
+      hi += v >> 32;
+      lo += int64_t(uint64_t(v) & 0xffffffffu);
+    }
+    int64_t *o = cols + (quarter * kTcBN + 32 * chunk + lane) * 2;
+    o[0] = hi;
+    o[1] = lo;
+  }
+  tc::tc_fence_before();
+  __syncthreads();
+  if (threadIdx.x < kTcBN) {
+    int64_t hi = 0, lo = 0;
+    for (int q = 0; q < 4; ++q) {
+      hi += cols[(q * kTcBN + threadIdx.x) * 2];
+      lo += cols[(q * kTcBN + threadIdx.x) * 2 + 1];
+    }
+    int64_t *o = part + size_t(blockIdx.y) * 2 * s.Cp + n0 + threadIdx.x;
+    o[0] = hi;
+    o[s.Cp] = lo;
+  }
+  if (warp == 0) {
+    tc::tc_fence_after();
+    tc::tmem_dealloc(tmem, 256);
+  }
+}
+
+// E_c = -2^(-k-1) (sum of the row blocks), one warp per column.
+__global__ void k_energy_fx_final(int C, int Cp, int blocks, int k, const int64_t *part, double *e) {
+  const int c = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  if (c >= C) return;
+  long long hi = 0, lo = 0;
+  for (int q = lane; q < blocks; q += 32) {
+    hi += part[size_t(q) * 2 * Cp + c];
+    lo += part[(size_t(q) * 2 + 1) * Cp + c];
+  }
+  for (int o = 16; o > 0; o >>= 1) {
+    hi += __shfl_down_sync(0xffffffffu, hi, o);
+    lo += __shfl_down_sync(0xffffffffu, lo, o);
+  }
+  if (lane == 0) {
+    hi += lo >> 32;  // now 0 <= lo < 2^32 and |hi| < 2^48: both exact in FP64
+    lo &= 0xffffffffll;
+    e[c] = -scalbn(fma(double(hi), 4294967296.0, double(lo)), -k - 1);
+  }
+}
+
+size_t fx_digit_bytes(int Kp) { return size_t(kFxDigits) * Kp * Kp * 2; }
+bool fx_eligible(int Kp) { return Kp <= kFxMaxKp; }
+
+cudaError_t fx_plan_make(void **plan, const double *J, const double *h, int N, int Kp, void *digits, int64_t *H,
+                         unsigned long long *scratch, cudaStream_t st) {
+  *plan = nullptr;
+  cudaError_t e = cudaFuncSetAttribute((const void *)k_energy_dense_fx, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       kFxSmem);
+  if (e == cudaSuccess) e = cudaMemsetAsync(scratch, 0, sizeof(*scratch), st);
+  if (e != cudaSuccess) return e;
+  k_fx_rowsum<<<N, 256, 0, st>>>(J, h, N, scratch);
+  double most = 0.0;
+  if ((e = cudaGetLastError()) != cudaSuccess ||
+      (e = cudaMemcpyAsync(&most, scratch, sizeof(most), cudaMemcpyDeviceToHost, st)) != cudaSuccess ||
+      (e = cudaStreamSynchronize(st)) != cudaSuccess)
+    return e;
+  if (!std::isfinite(most)) return cudaSuccess;  // row sums past the FP64 range: no plan
+  auto *p = new FxPlan();
+  p->k = most > 0.0 ? 61 - std::ilogb(most) : 0;  // row sums below 2^62 after scaling
+  p->H = H;
+  const size_t total = size_t(Kp) * Kp;
+  k_fx_digits<<<unsigned((total + 255) / 256), 256, 0, st>>>(J, h, N, Kp, p->k, static_cast<uint16_t *>(digits), H);
+  e = cudaGetLastError();
+  if (e == cudaSuccess && !tc_make_map(&p->A, digits, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, uint64_t(kFxDigits) * Kp,
+                                       uint64_t(Kp), 64, 128, CU_TENSOR_MAP_SWIZZLE_128B))
+    e = cudaErrorInvalidValue;
+  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+  if (e != cudaSuccess) {
+    delete p;
+    return e;
+  }
+  *plan = p;
+  return cudaSuccess;
+}
+
+void fx_plan_free(void *plan) { delete static_cast<FxPlan *>(plan); }
+
+cudaError_t launch_energy_partials_fx(const void *tc_plan, const void *fx_plan, const StateView &s, int Kp,
+                                      uint8_t *FT, int b, int *err, const BestView &best, cudaStream_t st) {
+  const auto *p = static_cast<const FxPlan *>(fx_plan);
+  k_sign_to_ft16<<<dim3(unsigned(Kp / 64), unsigned(s.Cp / 64)), 256, 0, st>>>(s, reinterpret_cast<uint16_t *>(FT), Kp,
+                                                                             b);
+  cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
+  const dim3 grid(unsigned(s.Cp / kTcBN), unsigned(Kp / kTcBM));
+  // the partial sums of 128 rows take 16 bytes, those of the FP64 kernel's 32 rows 8
+  int64_t *part = reinterpret_cast<int64_t *>(best.part_f64);
+  k_energy_dense_fx<<<grid, kFxThreads, kFxSmem, st>>>(p->A, static_cast<const TcMaps *>(tc_plan)->B, s, Kp, b, err,
+                                                       p->H, part);
+  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  k_energy_fx_final<<<unsigned((s.C + 7) / 8), 256, 0, st>>>(s.C, s.Cp, Kp / kTcBM, p->k, part, best.e_f64);
+  return cudaGetLastError();
+}
+
+}  // namespace sbqa

@@ -268,6 +268,12 @@ cudaError_t launch_energy_dense_tc(const void *plan, const StateView &s, int Kp,
   return launch_final(s, E, b, st);
 }
 
+cudaError_t launch_energy_dense_fx(const void *plan, const StateView &s, int Kp, uint8_t *FT, int buffer, int *err,
+                                   const EnergyView &E, const BestView &b, cudaStream_t st) {
+  const cudaError_t e = launch_sign(s, st);
+  return e != cudaSuccess ? e : launch_energy_partials_fx(plan, E.fx, s, Kp, FT, buffer, err, b, st);
+}
+
 // ---------------------------------------------------------------- best per run
 // One block per run: warp 0 takes the argmin over the Pr replicas (lowest k
 // on ties; replica k of run r is column r * P + k), kept if strictly lower
