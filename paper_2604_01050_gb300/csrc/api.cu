@@ -1888,7 +1888,7 @@ int sbqa_run(sbqa_problem *p, int32_t steps, int32_t P, int32_t R, uint64_t seed
       a.N = p->n; a.P = P; a.R = R; a.S = steps; a.Cp = p->Cp; a.seed = seed;
       a.amp = float(p->prm.init_amp); a.kc = p->tables.kc; a.kx = p->tables.kx;
       a.J = p->d_dense_f32.p; a.ka = p->d_ka.p; a.dl = p->d_dl.p; a.kj = p->d_kj.p; a.h = p->d_h.p;
-      a.J_i32 = p->d_e_i32.p; a.h_i64 = p->d_h_i64.p;
+      a.J_i32 = p->d_e_i32.p; a.max_abs_j = p->max_abs_j; a.h_i64 = p->d_h_i64.p;
       a.x = p->d_x.p; a.y = p->d_y.p; a.Sg = p->d_Sg.p; a.e_int = p->d_ei.p; a.e_f64 = p->d_ef.p;
       a.best_e_int = p->d_best_ei.p; a.best_e = p->d_best_e.p; a.best_k = p->d_best_k.p;
       a.best_step = p->d_best_step.p; a.have_best = p->d_have.p; a.best_spins = p->d_best_spins.p;

@@ -268,6 +268,7 @@ struct SmallArgs {
   const float *ka, *dl, *kj;
   const float *h;        // [N]
   const int32_t *J_i32;  // [N][N]
+  int max_abs_j;
   const int64_t *h_i64;  // [N]
   float *x, *y;          // [N][Cp]
   int8_t *Sg;
