@@ -1363,6 +1363,25 @@ int check_run_args(sbqa_problem *p, int32_t steps, int32_t P, int32_t R) {
   return SBQA_OK;
 }
 
+// The caller's state arrays [R * P][N] pass through the device in slices of
+// whole replicas (at most 32 MiB, one replica at least), where a kernel
+// changes the layout; the slice comes from the block cache and goes back to
+// it.  Its last words take two flags.
+struct StateSlices {
+  const sbqa_problem *p;
+  int replicas, per_slice;
+  DevBuf<float> rows;
+  explicit StateSlices(const sbqa_problem *q) : p(q), replicas(q->R * q->P) {
+    const int64_t fit = (int64_t(8) << 20) / std::max(1, q->n);
+    per_slice = int(std::max<int64_t>(1, std::min<int64_t>(fit, replicas)));
+  }
+  cudaError_t alloc() { return rows.alloc(size_t(per_slice) * p->n + 2); }
+  ~StateSlices() {
+    if (rows.p) cudaStreamSynchronize(p->stream);  // also after an error: nothing uses the slice any more
+    rows.release(true);
+  }
+};
+
 }  // namespace
 
 // ---- helpers shared with the batching engine (problem.h) ----
@@ -2002,18 +2021,18 @@ int sbqa_get_state(sbqa_problem *p, float *x, float *y, int32_t *step_done) {
   int rc = sbqa_synchronize(p);
   if (rc != SBQA_OK) return rc;
   DeviceGuard g(p->device);
-  const size_t NC = size_t(p->n) * p->Cp;
-  std::vector<float> buf(NC);
-  float *outs[2] = {x, y};
-  const float *src[2] = {p->d_x.p, p->d_y.p};
+  StateSlices sl(p);
+  SBQA_CUDA(sl.alloc());
+  float *outs[2] = {x, y}, *src[2] = {p->d_x.p, p->d_y.p};
   for (int w = 0; w < 2; ++w) {
     if (!outs[w]) continue;
-    SBQA_CUDA(cudaMemcpy(buf.data(), src[w], NC * sizeof(float), cudaMemcpyDeviceToHost));
-    for (int r = 0; r < p->R; ++r)
-      for (int k = 0; k < p->P; ++k) {
-        const size_t c = size_t(r) * p->Ps + k, o = (size_t(r) * p->P + k) * p->n;
-        for (int i = 0; i < p->n; ++i) outs[w][o + i] = buf[size_t(i) * p->Cp + c];
-      }
+    for (int q0 = 0; q0 < sl.replicas; q0 += sl.per_slice) {
+      const int count = std::min(sl.per_slice, sl.replicas - q0);
+      SBQA_CUDA(launch_state_rows(p->state(), src[w], sl.rows.p, q0, count, true, nullptr, p->stream));
+      SBQA_CUDA(cudaMemcpyAsync(outs[w] + size_t(q0) * p->n, sl.rows.p, size_t(count) * p->n * sizeof(float),
+                                cudaMemcpyDeviceToHost, p->stream));
+      SBQA_CUDA(cudaStreamSynchronize(p->stream));
+    }
   }
   if (step_done) *step_done = p->step_done;
   return SBQA_OK;
@@ -2026,20 +2045,27 @@ int sbqa_set_state(sbqa_problem *p, const float *x, const float *y, int32_t step
   int rc = sbqa_synchronize(p);
   if (rc != SBQA_OK) return rc;
   DeviceGuard g(p->device);
+  StateSlices sl(p);
+  SBQA_CUDA(sl.alloc());
   const size_t NC = size_t(p->n) * p->Cp;
-  std::vector<float> bx(NC, 0.f), by(NC, 0.f);  // padding columns of a run stay at zero
-  for (int r = 0; r < p->R; ++r)
-    for (int k = 0; k < p->P; ++k) {
-      const size_t c = size_t(r) * p->Ps + k, o = (size_t(r) * p->P + k) * p->n;
-      for (int i = 0; i < p->n; ++i) {
-        bx[size_t(i) * p->Cp + c] = x[o + i];
-        by[size_t(i) * p->Cp + c] = y[o + i];
-      }
+  const float *in[2] = {x, y};
+  float *dst[2] = {p->d_x.p, p->d_y.p};
+  int *wide = reinterpret_cast<int *>(sl.rows.p + size_t(sl.per_slice) * p->n);  // of x, then of y
+  int is_wide[2] = {0, 0};
+  SBQA_CUDA(cudaMemsetAsync(wide, 0, sizeof(is_wide), p->stream));
+  for (int w = 0; w < 2; ++w) {
+    SBQA_CUDA(cudaMemsetAsync(dst[w], 0, NC * sizeof(float), p->stream));  // padding columns of a run stay at zero
+    for (int q0 = 0; q0 < sl.replicas; q0 += sl.per_slice) {
+      const int count = std::min(sl.per_slice, sl.replicas - q0);
+      SBQA_CUDA(cudaMemcpyAsync(sl.rows.p, in[w] + size_t(q0) * p->n, size_t(count) * p->n * sizeof(float),
+                                cudaMemcpyHostToDevice, p->stream));
+      SBQA_CUDA(launch_state_rows(p->state(), dst[w], sl.rows.p, q0, count, false, wide + w, p->stream));
+      SBQA_CUDA(cudaStreamSynchronize(p->stream));
     }
-  p->wide_x = false;
-  for (float v : bx) p->wide_x = p->wide_x || !(std::fabs(v) < 2.f);
-  SBQA_CUDA(cudaMemcpy(p->d_x.p, bx.data(), NC * sizeof(float), cudaMemcpyHostToDevice));
-  SBQA_CUDA(cudaMemcpy(p->d_y.p, by.data(), NC * sizeof(float), cudaMemcpyHostToDevice));
+  }
+  SBQA_CUDA(cudaMemcpyAsync(is_wide, wide, sizeof(is_wide), cudaMemcpyDeviceToHost, p->stream));
+  SBQA_CUDA(cudaStreamSynchronize(p->stream));
+  p->wide_x = is_wide[0] != 0;
   const double tau = p->S > 0 ? double(step_done) / double(p->S) : 0.0;
   SBQA_CUDA(launch_refresh_f(p->state(), step_done & 1, float(p->prm.delta_slope * tau), p->stream));
   if (p->use_tc)

@@ -101,3 +101,16 @@ def test_ballistic_states_from_outside_the_wall(sb, value):
         out.append(sb.get_state(pb))
     assert np.array_equal(out[0][0], out[1][0]) and np.array_equal(out[0][1], out[1][1])
 
+
+@pytest.mark.parametrize("N,P,R", [(1, 1, 1), (31, 3, 5), (33, 7, 9), (216, 12, 3), (1000, 64, 2)])
+def test_state_round_trip(sb, N, P, R):
+    """get_state and set_state in the caller's layout: what goes in comes out, padding untouched."""
+    J = np.zeros((N, N))
+    pb = sb.create_problem_dense(J)
+    sb.set_schedule(pb, *workloads.autotune_params(R, 1))
+    sb.run_begin(pb, 10, P, R, seed=5)
+    rng = np.random.default_rng(N)
+    x, y = (rng.uniform(-1, 1, (R, P, N)).astype(np.float32) for _ in range(2))
+    sb.set_state(pb, x, y, 4)
+    x2, y2, done = sb.get_state(pb)
+    assert done == 4 and np.array_equal(x, x2) and np.array_equal(y, y2)
