@@ -11,8 +11,7 @@
 //   k_step_csr_bsb    one warp per (spin row, 128 replica columns), 4 columns
 //                     per lane; 8 neighbour gathers (16 bytes each) in flight;
 //                     FP32 accumulation in the row's CSR order
-//   k_step_dense_bsb  32 rows x 128 columns per block; J (FP32) and x (FP32)
-//                     tiles staged in shared memory
+//   (dense J: k_step_dense in step_dense.cu)
 // Memory per update: x, y read + write (16 B) + f write (4 B); the gathers of
 // neighbour f (4 B per coupling) mostly hit in L2.
 #include "step_common.cuh"
@@ -69,68 +68,6 @@ __global__ void __launch_bounds__(256) k_step_csr_bsb(StateView s, CsrView J, St
   sb_update4_bsb<P>(s, t, n, i, c4, g, __ldg(J.h + i), xv, yv, s.fx_of(n + 1));
 }
 
-constexpr int kBsbBM = 32, kBsbBK = 32;
-
-template <int P>
-__global__ void __launch_bounds__(256) k_step_dense_bsb(StateView s, DenseView J, StepTables t, int n) {
-  __shared__ float Js[kBsbBM][kBsbBK + 1];
-  __shared__ __align__(16) float Fs[kBsbBK][kColsPerWarp];
-  const int row0 = blockIdx.y * kBsbBM;
-  const int col0 = blockIdx.x * kColsPerWarp;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const float *Fin = s.fx_of(n);
-  const int N = s.N;
-  float acc[4][4];
-#pragma unroll
-  for (int a = 0; a < 4; ++a)
-#pragma unroll
-    for (int b = 0; b < 4; ++b) acc[a][b] = 0.f;
-  for (int k0 = 0; k0 < N; k0 += kBsbBK) {
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {  // J tile: 1024 floats, 4 per thread
-      const int idx = threadIdx.x + q * 256;
-      const int r = idx >> 5, k = idx & 31;
-      const int gi = row0 + r, gk = k0 + k;
-      Js[r][k] = (gi < N && gk < N) ? __ldg(J.J + size_t(gi) * N + gk) : 0.f;
-    }
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {  // f tile: 32 rows x 128 floats, 4 float4 per thread
-      const int idx = threadIdx.x + q * 256;
-      const int r = idx >> 5, seg = (idx & 31) * 4;
-      const int gk = k0 + r;
-      float4 v = make_float4(0.f, 0.f, 0.f, 0.f);  // f = 0 past the last spin
-      if (gk < N) v = __ldg(reinterpret_cast<const float4 *>(Fin + size_t(gk) * s.Cp + col0 + seg));
-      *reinterpret_cast<float4 *>(&Fs[r][seg]) = v;
-    }
-    __syncthreads();
-#pragma unroll 8
-    for (int k = 0; k < kBsbBK; ++k) {
-      const float4 f = *reinterpret_cast<const float4 *>(&Fs[k][lane * 4]);
-#pragma unroll
-      for (int a = 0; a < 4; ++a) {
-        const float w = Js[warp * 4 + a][k];
-        acc[a][0] = fmaf(w, f.x, acc[a][0]);
-        acc[a][1] = fmaf(w, f.y, acc[a][1]);
-        acc[a][2] = fmaf(w, f.z, acc[a][2]);
-        acc[a][3] = fmaf(w, f.w, acc[a][3]);
-      }
-    }
-    __syncthreads();
-  }
-  const int c4 = col0 + lane * 4;
-  float *Fout = s.fx_of(n + 1);
-#pragma unroll
-  for (int a = 0; a < 4; ++a) {
-    const int i = row0 + warp * 4 + a;
-    if (i < N) {
-      const size_t off = size_t(i) * s.Cp + c4;
-      const float4 xv = *reinterpret_cast<const float4 *>(s.x + off);
-      const float4 yv = *reinterpret_cast<const float4 *>(s.y + off);
-      sb_update4_bsb<P>(s, t, n, i, c4, acc[a], __ldg(J.h + i), xv, yv, Fout);
-    }
-  }
-}
-
 __global__ void k_copy_fx(const float *x, float *fx, size_t count) {
   const size_t e = size_t(blockIdx.x) * blockDim.x + threadIdx.x;
   if (e < count) fx[e] = x[e];
@@ -147,14 +84,6 @@ static cudaError_t launch_csr_p(const StateView &s, const CsrView &J, const Step
   return cudaGetLastError();
 }
 
-template <int P>
-static cudaError_t launch_dense_p(const StateView &s, const DenseView &J, const StepTables &t, int n,
-                                  cudaStream_t st) {
-  const dim3 grid(unsigned(s.Cp / kColsPerWarp), unsigned((s.N + kBsbBM - 1) / kBsbBM));
-  k_step_dense_bsb<P><<<grid, 256, 0, st>>>(s, J, t, n);
-  return cudaGetLastError();
-}
-
 cudaError_t launch_step_csr_bsb(const StateView &s, const CsrView &J, const StepTables &t, int n, cudaStream_t st) {
   switch (s.P) {
     case 1: return launch_csr_p<1>(s, J, t, n, st);
@@ -165,21 +94,6 @@ cudaError_t launch_step_csr_bsb(const StateView &s, const CsrView &J, const Step
     case 32: return launch_csr_p<32>(s, J, t, n, st);
     case 64: return launch_csr_p<64>(s, J, t, n, st);
     case 128: return launch_csr_p<128>(s, J, t, n, st);
-    default: return cudaErrorInvalidValue;
-  }
-}
-
-cudaError_t launch_step_dense_bsb(const StateView &s, const DenseView &J, const StepTables &t, int n,
-                                  cudaStream_t st) {
-  switch (s.P) {
-    case 1: return launch_dense_p<1>(s, J, t, n, st);
-    case 2: return launch_dense_p<2>(s, J, t, n, st);
-    case 4: return launch_dense_p<4>(s, J, t, n, st);
-    case 8: return launch_dense_p<8>(s, J, t, n, st);
-    case 16: return launch_dense_p<16>(s, J, t, n, st);
-    case 32: return launch_dense_p<32>(s, J, t, n, st);
-    case 64: return launch_dense_p<64>(s, J, t, n, st);
-    case 128: return launch_dense_p<128>(s, J, t, n, st);
     default: return cudaErrorInvalidValue;
   }
 }
