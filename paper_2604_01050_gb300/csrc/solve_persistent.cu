@@ -1,6 +1,7 @@
 // solve_persistent.cu -- all steps of a CSR run batch in one cooperative launch.
 //
-// For rows of degree <= 8 (+-1, FP32 or BF16 couplings).  One block of 32
+// For rows of degree <= 32 (+-1, FP32 or BF16 couplings; up to 8 for the
+// ballistic form, whose lists and the streaming form's are of 8 slots).  One block of 32
 // warps per SM; every warp owns fixed work items (spin row, 128 or 256
 // replica columns) for the whole launch -- individual items, or whole rows
 // with all their chunks when the items outnumber the cache.  A pass is what
@@ -28,6 +29,8 @@
 //   lattice L = 16, R*P = 2048     24.0 -> 13.3    random graph N = 10^5,
 //   lattice L = 10, R*P = 1024      4.9 ->  3.1    R*P = 128, BF16 46.8 -> 27.8
 //   lattice L = 24, R*P = 2048     81.9 -> 70.2    N = 3000 3.0 -> 2.0
+//   degree 12 (per-step kernels before), N = 20000, R*P = 128, FP32 13.9 -> 8.5
+//   degree 20, N = 3001, R*P = 160 6.1 -> 4.4; N = 60000, R*P = 128 52.8 -> 35.9
 //   ballistic L = 16 36.6 -> 32.0, L = 12, R*P = 512 5.6 -> 3.8, N = 10^5 61.8 -> 55.3
 //
 // Per pass a warp gathers the codes of the (at most 8) neighbours, sums (same
@@ -59,7 +62,9 @@
 
 namespace sbqa {
 
-constexpr int kPersistMaxDeg = 8;
+constexpr int kPersistMaxDeg = 8;    // slots of the short lists
+constexpr int kPersistWideDeg = 32;  // and of the long ones
+constexpr int kWideAtOnce = 12;      // slots of a long list gathered at a time (24 registers of codes; 32 spill)
 constexpr int kPersistWarps = 24, kPersistThreads = 32 * kPersistWarps;
 constexpr int kPersistSmem = 225 * 1024;               // dynamic shared memory of a block
 constexpr int kWarpSmem = kPersistSmem / kPersistWarps;  // 9600 bytes per warp
@@ -81,6 +86,8 @@ struct PersistArgs {
   // ELL form of the couplings (rows of degree <= 8, the CSR kernels' entry order)
   const int32_t *ell_col, *ell_meta;
   const float *ell_val;
+  CsrView csr;    // the long lists are filled from the CSR arrays
+  int wide;       // slots of a long list (degree rounded up to a multiple of 4)
   StepTables t;
   int n_begin, n_end;
   int *err;       // error flag
@@ -127,6 +134,51 @@ struct WarpCache {
         reinterpret_cast<int8_t *>(vals)[8 * q + lane] = used ? (lane < m.y ? 1 : -1) : 0;
     } else if (lane == kPersistMaxDeg) {
       meta[q] = uint32_t(m.x) | (uint32_t(2 * m.y - m.x) << 16);
+      item[q] = make_int2(row, chunk);
+    }
+  }
+};
+
+// The same for rows of up to 32 entries: lists of W slots (a multiple of 4),
+// filled from the CSR arrays a slot per lane.
+constexpr int wide_bytes(int W, bool vals) { return 4 * W + (vals ? 4 * W : W) + 12; }
+
+template <bool VALS>
+struct WideCache {
+  int4 *cols;      // [cap][W / 4]
+  float4 *vals;    // [cap][W / 4]
+  int2 *item;      // [cap] (row, chunk)
+  uint32_t *meta;  // [cap] degree | (sum of signs) << 16
+  uint32_t *signs;  // [cap][W / 4] signed bytes
+  int W;
+  __device__ WideCache(char *base, int cap, int w) : W(w) {
+    cols = reinterpret_cast<int4 *>(base);
+    base += 4 * W * cap;
+    vals = reinterpret_cast<float4 *>(base);
+    if (VALS) base += 4 * W * cap;
+    item = reinterpret_cast<int2 *>(base);
+    base += 8 * cap;
+    meta = reinterpret_cast<uint32_t *>(base);
+    signs = meta + cap;
+  }
+  __device__ __forceinline__ void fill(const PersistArgs &a, int q, int row, int chunk, int lane) const {
+    const int e0 = __ldg(a.csr.row_ptr + row), deg = __ldg(a.csr.row_ptr + row + 1) - e0;
+    const int pos = VALS ? deg : __ldg(a.csr.npos + row);
+    if (lane < W) {
+      const bool used = lane < deg;
+      reinterpret_cast<int32_t *>(cols)[W * q + lane] = used ? __ldg(a.csr.col + e0 + lane) : row;
+      if constexpr (VALS) {
+        float v = 0.f;
+        if (used)
+          v = a.csr.kind == VAL_BF16 ? __bfloat162float(static_cast<const __nv_bfloat16 *>(a.csr.val)[e0 + lane])
+                                     : static_cast<const float *>(a.csr.val)[e0 + lane];
+        reinterpret_cast<float *>(vals)[W * q + lane] = v;
+      } else {
+        reinterpret_cast<int8_t *>(signs)[W * q + lane] = used ? (lane < pos ? 1 : -1) : 0;
+      }
+    }
+    if (lane == 0) {
+      meta[q] = uint32_t(deg) | (uint32_t(2 * pos - deg) << 16);
       item[q] = make_int2(row, chunk);
     }
   }
@@ -180,6 +232,30 @@ __device__ __forceinline__ bool wait_over(unsigned it, uint64_t &t0, int *err) {
   return true;
 }
 
+// Packed sums of sign * code of four columns a word: per byte 64 + the sum over
+// the entries, between 0 and 128 for up to 32 of them.
+__device__ __forceinline__ uint32_t packed_start(uint32_t tag, int sum) { return 0x40404040u - tag * uint32_t(sum); }
+__device__ __forceinline__ void add_signed(uint32_t (&acc)[2], const Codes8 &f, uint32_t signs, int byte) {
+  const uint32_t b = uint32_t(byte);
+  uint32_t sign;  // the byte, sign extended
+  asm("prmt.b32 %0, %1, 0, %2;" : "=r"(sign) : "r"(signs), "r"(b | (0x888u | b * 0x111u) << 4));
+  acc[0] += sign * f.w[0];
+  acc[1] += sign * f.w[1];
+}
+__device__ __forceinline__ void packed_finish(const uint32_t (&acc)[2], int sum, float (&G)[8]) {
+  const float off = -8388608.f - float(64 + sum);
+#pragma unroll
+  for (int c = 0; c < 8; c += 2) {
+    const uint32_t m0 = __byte_perm(acc[c / 4], 0x4B000000u, 0x7540u | uint32_t(c % 4));
+    const uint32_t m1 = __byte_perm(acc[c / 4], 0x4B000000u, 0x7540u | uint32_t(c % 4 + 1));
+    const float2 g = __fadd2_rn(make_float2(__uint_as_float(m0), __uint_as_float(m1)), make_float2(off, off));
+    G[c] = g.x;
+    G[c + 1] = g.y;
+  }
+}
+// -(2^23 + 1), and the generation bit of a code read through the low mantissa bits of 2^23
+__device__ __forceinline__ float code_offset(uint32_t tag) { return tag ? -8388737.f : -8388609.f; }
+
 // Coupling sums of one pass from the gathered codes of the lane's 8 columns
 // (with their generation bits).  +-1: packed sums of sign * code -- integers
 // modulo 2^32, so the bits and the offset codes carry are taken out at the
@@ -194,16 +270,9 @@ __device__ __forceinline__ void sum_codes(const Codes8 (&f)[kPersistMaxDeg], uin
   if constexpr (KIND == VAL_PM1) {
     const int2 sg = *reinterpret_cast<const int2 *>(vals);
     const int sum = int(meta) >> 16;
-    // per byte: 64 + sum over entries of sign * code, between 48 and 80
     uint32_t acc[2];
-    acc[0] = acc[1] = 0x40404040u - tag * uint32_t(sum);
-    auto add = [&](int e) {
-      const uint32_t b = uint32_t(e & 3), w = uint32_t(e < 4 ? sg.x : sg.y);
-      uint32_t sign;  // byte b, sign extended
-      asm("prmt.b32 %0, %1, 0, %2;" : "=r"(sign) : "r"(w), "r"(b | (0x888u | b * 0x111u) << 4));
-      acc[0] += sign * f[e].w[0];
-      acc[1] += sign * f[e].w[1];
-    };
+    acc[0] = acc[1] = packed_start(tag, sum);
+    auto add = [&](int e) { add_signed(acc, f[e], uint32_t(e < 4 ? sg.x : sg.y), e & 3); };
 #pragma unroll
     for (int e = 0; e < 4; ++e) add(e);
     if (slots > 4) {
@@ -214,19 +283,11 @@ __device__ __forceinline__ void sum_codes(const Codes8 (&f)[kPersistMaxDeg], uin
       add(6);
       add(7);
     }
-    const float off = -8388608.f - float(64 + sum);
-#pragma unroll
-    for (int c = 0; c < 8; c += 2) {
-      const uint32_t m0 = __byte_perm(acc[c / 4], 0x4B000000u, 0x7540u | uint32_t(c % 4));
-      const uint32_t m1 = __byte_perm(acc[c / 4], 0x4B000000u, 0x7540u | uint32_t(c % 4 + 1));
-      const float2 g = __fadd2_rn(make_float2(__uint_as_float(m0), __uint_as_float(m1)), make_float2(off, off));
-      G[c] = g.x;
-      G[c + 1] = g.y;
-    }
+    packed_finish(acc, sum, G);
   } else {
 #pragma unroll
     for (int c = 0; c < 8; ++c) G[c] = 0.f;
-    const float off = tag ? -8388737.f : -8388609.f;  // -(2^23 + 1), and the generation bit
+    const float off = code_offset(tag);
     const float4 v = vals[0];
     acc_codes_off<8>(G, v.x, f[0].w, off);
     acc_codes_off<8>(G, v.y, f[1].w, off);
@@ -264,7 +325,8 @@ __device__ __forceinline__ bool codes_fresh(const Codes8 (&f)[kPersistMaxDeg], u
 }
 
 // LPI = 32: passes of one 256-column item on the whole warp; 16: of two 128-column ones on half warps.
-template <int P, int KIND, int LPI>
+// WIDE: lists of up to 32 slots, gathered and summed 12 at a time.
+template <int P, int KIND, int LPI, bool WIDE>
 __global__ void __launch_bounds__(kPersistThreads, 1) k_solve_csr_persistent(PersistArgs a) {
   constexpr bool VALS = KIND != VAL_PM1;
   constexpr int IPW = 32 / LPI;  // items per pass
@@ -277,7 +339,10 @@ __global__ void __launch_bounds__(kPersistThreads, 1) k_solve_csr_persistent(Per
   const int gw = blockIdx.x * kPersistWarps + warp;
   char *mine = s_raw + warp * a.warp_smem;
   float4 *state = reinterpret_cast<float4 *>(mine);  // [slots][x lo, x hi, y lo, y hi][lane]
-  const WarpCache<VALS> cache(mine + a.slots * kSlotBytes, a.cache_cap);
+  const auto cache = [&] {
+    if constexpr (WIDE) return WideCache<VALS>(mine + a.slots * kSlotBytes, a.cache_cap, a.wide);
+    else return WarpCache<VALS>(mine + a.slots * kSlotBytes, a.cache_cap);
+  }();
   if (warp == 0) tc::tmem_alloc(&s_tmem, kPersistTmem);
   int my_count = 0;
   const int n_units = s.N * chunks;
@@ -384,6 +449,63 @@ __global__ void __launch_bounds__(kPersistThreads, 1) k_solve_csr_persistent(Per
       gather(f, n, cols, c0);
     }
   };
+  // Coupling sums of a long list; false when the warp gave up.
+  auto wide_sums = [&](int n, const Pass &t, uint32_t tag, float (&G)[8]) {
+    if constexpr (WIDE) {
+      const uint8_t *F = s.f_of(n) + t.c0;
+      const int W4 = a.wide / 4, sum = int(cache.meta[t.e]) >> 16;
+      uint32_t acc[2];
+      acc[0] = acc[1] = packed_start(tag, sum);
+#pragma unroll
+      for (int c = 0; c < 8; ++c) G[c] = 0.f;
+      const float coff = code_offset(tag);
+      for (int g0 = 0; g0 < W4; g0 += kWideAtOnce / 4) {
+        const int4 *cols = cache.cols + W4 * t.e + g0;
+        Codes8 f[kWideAtOnce];
+        uint64_t t0 = 0;
+        for (unsigned it = 0;; ++it) {  // until every live lane's codes are of step n
+#pragma unroll
+          for (int g = 0; g < kWideAtOnce / 4; ++g)
+            if (g0 + g < W4) {
+              const int4 c = cols[g];
+              f[4 * g].load(F + size_t(c.x) * s.Cp);
+              f[4 * g + 1].load(F + size_t(c.y) * s.Cp);
+              f[4 * g + 2].load(F + size_t(c.z) * s.Cp);
+              f[4 * g + 3].load(F + size_t(c.w) * s.Cp);
+            }
+          uint32_t all = ~0u, any = 0u;
+#pragma unroll
+          for (int g = 0; g < kWideAtOnce / 4; ++g)
+            if (g0 + g < W4)
+#pragma unroll
+              for (int u = 0; u < 4; ++u) {
+                if (tag) all &= f[4 * g + u].w[0] & f[4 * g + u].w[1];
+                else any |= f[4 * g + u].w[0] | f[4 * g + u].w[1];
+              }
+          const bool stale = tag ? (all & kTagCodes) != kTagCodes : (any & kTagCodes) != 0;
+          if (!__any_sync(0xffffffffu, t.live && stale) || n == a.n_begin) break;
+          if (wait_over(it, t0, a.err)) return false;
+        }
+#pragma unroll
+        for (int g = 0; g < kWideAtOnce / 4; ++g)
+          if (g0 + g < W4) {
+            if constexpr (VALS) {
+              const float4 v = cache.vals[W4 * t.e + g0 + g];
+              acc_codes_off<8>(G, v.x, f[4 * g].w, coff);
+              acc_codes_off<8>(G, v.y, f[4 * g + 1].w, coff);
+              acc_codes_off<8>(G, v.z, f[4 * g + 2].w, coff);
+              acc_codes_off<8>(G, v.w, f[4 * g + 3].w, coff);
+            } else {
+              const uint32_t sg = cache.signs[W4 * t.e + g0 + g];
+#pragma unroll
+              for (int u = 0; u < 4; ++u) add_signed(acc, f[4 * g + u], sg, u);
+            }
+          }
+      }
+      if constexpr (!VALS) packed_finish(acc, sum, G);
+    }
+    return true;
+  };
   // Update of one pass from its coupling sums; slot < 0: the state is in xs, ys and goes back to
   // global memory, else it lives on the chip in that slot.
   auto update = [&](int n, const Pass &t, int slot, const float (&G)[8], const float (&kj)[P >= 8 ? 1 : 8 / P],
@@ -417,20 +539,31 @@ __global__ void __launch_bounds__(kPersistThreads, 1) k_solve_csr_persistent(Per
     for (int p = 0; p < passes; ++p) {
       const Pass t = locate(p);
       float xs[8], ys[8], G[8], kj[P >= 8 ? 1 : 8 / P];
-      if (p >= resident) {
-        const size_t off = size_t(t.i) * s.Cp + t.c0;
-        load_row_now(s.x + off, xs);
-        load_row_now(s.y + off, ys);
+      const size_t off = size_t(t.i) * s.Cp + t.c0;
+      float hi;
+      if constexpr (!WIDE) {
+        if (p >= resident) {
+          load_row_now(s.x + off, xs);
+          load_row_now(s.y + off, ys);
+        }
+        Codes8 f[kPersistMaxDeg];
+        const int4 *cols = cache.cols + 2 * t.e;
+        gather(f, n, cols, t.c0);
+        load_kj<P, 8>(kjn, s.C, t.c0, kj);
+        hi = __ldg(a.h + t.i);
+        if (!(ok = fresh(f, n, cols, t.c0, t.live, tag))) break;
+        sum_codes<KIND>(f, tag, VALS ? cache.vals + 2 * t.e : reinterpret_cast<const float4 *>(
+                                                                  reinterpret_cast<const int2 *>(cache.vals) + t.e),
+                        cache.meta[t.e], a.degree, G);
+      } else {
+        if (!(ok = wide_sums(n, t, tag, G))) break;
+        if (p >= resident) {
+          load_row_now(s.x + off, xs);
+          load_row_now(s.y + off, ys);
+        }
+        load_kj<P, 8>(kjn, s.C, t.c0, kj);
+        hi = __ldg(a.h + t.i);
       }
-      Codes8 f[kPersistMaxDeg];
-      const int4 *cols = cache.cols + 2 * t.e;
-      gather(f, n, cols, t.c0);
-      load_kj<P, 8>(kjn, s.C, t.c0, kj);
-      const float hi = __ldg(a.h + t.i);
-      if (!(ok = fresh(f, n, cols, t.c0, t.live, tag))) break;
-      sum_codes<KIND>(f, tag, VALS ? cache.vals + 2 * t.e : reinterpret_cast<const float4 *>(
-                                                                reinterpret_cast<const int2 *>(cache.vals) + t.e),
-                      cache.meta[t.e], a.degree, G);
       update(n, t, p < resident ? p : -1, G, kj, hi, ka, dnext, xs, ys);
     }
   }
@@ -652,24 +785,29 @@ static const void *persistent_bsb_fn(int P, int kind) {
   return kind == VAL_PM1 ? persistent_bsb_fn_k<VAL_PM1>(P) : persistent_bsb_fn_k<VAL_F32>(P);
 }
 
-template <int KIND, int LPI>
+template <int KIND, int LPI, bool WIDE>
 static const void *persistent_fn_p(int P) {
   switch (P) {
-    case 1: return (const void *)k_solve_csr_persistent<1, KIND, LPI>;
-    case 2: return (const void *)k_solve_csr_persistent<2, KIND, LPI>;
-    case 4: return (const void *)k_solve_csr_persistent<4, KIND, LPI>;
-    case 8: return (const void *)k_solve_csr_persistent<8, KIND, LPI>;
-    case 16: return (const void *)k_solve_csr_persistent<16, KIND, LPI>;
-    case 32: return (const void *)k_solve_csr_persistent<32, KIND, LPI>;
-    case 64: return (const void *)k_solve_csr_persistent<64, KIND, LPI>;
-    case 128: return (const void *)k_solve_csr_persistent<128, KIND, LPI>;
+    case 1: return (const void *)k_solve_csr_persistent<1, KIND, LPI, WIDE>;
+    case 2: return (const void *)k_solve_csr_persistent<2, KIND, LPI, WIDE>;
+    case 4: return (const void *)k_solve_csr_persistent<4, KIND, LPI, WIDE>;
+    case 8: return (const void *)k_solve_csr_persistent<8, KIND, LPI, WIDE>;
+    case 16: return (const void *)k_solve_csr_persistent<16, KIND, LPI, WIDE>;
+    case 32: return (const void *)k_solve_csr_persistent<32, KIND, LPI, WIDE>;
+    case 64: return (const void *)k_solve_csr_persistent<64, KIND, LPI, WIDE>;
+    case 128: return (const void *)k_solve_csr_persistent<128, KIND, LPI, WIDE>;
     default: return nullptr;
   }
 }
 
-static const void *persistent_fn(int P, int kind, int lpi) {
-  if (kind == VAL_PM1) return lpi == 32 ? persistent_fn_p<VAL_PM1, 32>(P) : persistent_fn_p<VAL_PM1, 16>(P);
-  return lpi == 32 ? persistent_fn_p<VAL_F32, 32>(P) : persistent_fn_p<VAL_F32, 16>(P);
+template <bool WIDE>
+static const void *persistent_fn_k(int P, int kind, int lpi) {
+  if (kind == VAL_PM1) return lpi == 32 ? persistent_fn_p<VAL_PM1, 32, WIDE>(P) : persistent_fn_p<VAL_PM1, 16, WIDE>(P);
+  return lpi == 32 ? persistent_fn_p<VAL_F32, 32, WIDE>(P) : persistent_fn_p<VAL_F32, 16, WIDE>(P);
+}
+
+static const void *persistent_fn(int P, int kind, int lpi, bool wide) {
+  return wide ? persistent_fn_k<true>(P, kind, lpi) : persistent_fn_k<false>(P, kind, lpi);
 }
 
 // Items of 256 columns on whole warps when R * P allows it, else of 128 on half warps.
@@ -699,9 +837,11 @@ int persistent_blocks() {
   };
   const int Ps[8] = {1, 2, 4, 8, 16, 32, 64, 128};
   for (int P : Ps)
-    for (int kind : {VAL_PM1, VAL_F32})
-      if (!fits(persistent_fn(P, kind, 16)) || !fits(persistent_fn(P, kind, 32)) || !fits(persistent_bsb_fn(P, kind)))
-        return 0;
+    for (int kind : {VAL_PM1, VAL_F32}) {
+      for (int wide = 0; wide < 2; ++wide)
+        if (!fits(persistent_fn(P, kind, 16, wide != 0)) || !fits(persistent_fn(P, kind, 32, wide != 0))) return 0;
+      if (!fits(persistent_bsb_fn(P, kind))) return 0;
+    }
   return streaming_fits() ? sms : 0;
 }
 
@@ -745,7 +885,9 @@ static PersistArgs persist_args(const StateView &s, const CsrView &J, const Step
   // keep the codes of step n of a launch that runs it (not for production use)
   const char *skip = std::getenv("SBQA_TEST_SKIP_BARRIER_STEP");
   a.skip_step = skip ? std::atoi(skip) : -1;
+  a.csr = J;
   a.degree = J.max_degree;
+  a.wide = (J.max_degree + 3) / 4 * 4;
   a.cache_cap = a.slots = a.warp_smem = 0;
   return a;
 }
@@ -754,7 +896,11 @@ static PersistArgs persist_args(const StateView &s, const CsrView &J, const Step
 // generation bits is left from an earlier launch.
 static cudaError_t launch_persist(const void *fn, PersistArgs &a, int kind, void *other, size_t bytes, int blocks,
                                   cudaStream_t st) {
-  if (!fn || !a.ell_col || !a.ell_meta || (kind != VAL_PM1 && !a.ell_val)) return cudaErrorInvalidValue;
+  const bool lists = a.degree > kPersistMaxDeg
+                         ? a.csr.row_ptr && a.csr.col &&
+                               (kind == VAL_PM1 ? a.csr.npos != nullptr : a.csr.val != nullptr)
+                         : a.ell_col && a.ell_meta && (kind == VAL_PM1 || a.ell_val);
+  if (!fn || !lists) return cudaErrorInvalidValue;
   const cudaError_t e = cudaMemsetAsync(other, 0, bytes, st);
   if (e != cudaSuccess) return e;
   void *args[] = {&a};
@@ -775,11 +921,13 @@ cudaError_t launch_solve_csr_persistent_bsb(const StateView &s, const CsrView &J
 
 int persistent_mode(int N, int Cp, int max_degree, int kind, int blocks, bool force_rows, bool ell) {
   const int lpi = persist_lpi(Cp);
-  if (blocks <= 0 || max_degree > kPersistMaxDeg || lpi == 0 || !ell) return 0;
+  const bool wide = max_degree > kPersistMaxDeg;
+  if (blocks <= 0 || max_degree > kPersistWideDeg || lpi == 0 || (!wide && !ell)) return 0;
   const long long items = (long long)N * (Cp / (8 * lpi)), warps = (long long)blocks * kPersistWarps;
-  const long long most = std::min<long long>(kMaxPasses * (32 / lpi), cache_cap_hook());
+  long long most = std::min<long long>(kMaxPasses * (32 / lpi), cache_cap_hook());
+  if (wide) most = std::min<long long>(most, kWarpSmem / wide_bytes((max_degree + 3) / 4 * 4, kind != VAL_PM1));
   if (!force_rows && items <= warps * most) return kPersistResident;
-  return streaming_mode(N, Cp, max_degree, kind, blocks * kStreamBlocksPerSm, force_rows, ell);
+  return wide ? 0 : streaming_mode(N, Cp, max_degree, kind, blocks * kStreamBlocksPerSm, force_rows, ell);
 }
 
 cudaError_t launch_solve_csr_persistent(const StateView &s, const CsrView &J, const StepTables &t, int n_begin,
@@ -788,10 +936,11 @@ cudaError_t launch_solve_csr_persistent(const StateView &s, const CsrView &J, co
   if (mode != kPersistResident)
     return launch_solve_csr_streaming(s, J, t, n_begin, n_end, bar, err, blocks * kStreamBlocksPerSm, mode, st);
   PersistArgs a = persist_args(s, J, t, n_begin, n_end, err);
-  split_smem(&a, (long long)s.N * (s.Cp / (8 * lpi)), blocks * kPersistWarps, entry_bytes(J.kind != VAL_PM1), 32 / lpi,
-             kTmemPasses, kSlotBytes);
-  return launch_persist(persistent_fn(s.P, J.kind, lpi), a, J.kind, s.f_of(n_begin + 1), size_t(s.N) * s.Cp, blocks,
-                        st);
+  const bool vals = J.kind != VAL_PM1, wide = J.max_degree > kPersistMaxDeg;
+  split_smem(&a, (long long)s.N * (s.Cp / (8 * lpi)), blocks * kPersistWarps,
+             wide ? wide_bytes(a.wide, vals) : entry_bytes(vals), 32 / lpi, kTmemPasses, kSlotBytes);
+  return launch_persist(persistent_fn(s.P, J.kind, lpi, wide), a, J.kind, s.f_of(n_begin + 1), size_t(s.N) * s.Cp,
+                        blocks, st);
 }
 
 }  // namespace sbqa

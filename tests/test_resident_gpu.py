@@ -60,6 +60,37 @@ def test_resident_equals_per_step(sb, name, variant):
     assert np.array_equal(a[4][0], b[4][0]) and np.array_equal(a[4][1], b[4][1])
 
 
+def _signs(spec):
+    kind, n, rp, col, val, _ = spec
+    return kind, n, rp, col, np.where(val > 0, 1.0, -1.0), None
+
+
+@pytest.mark.parametrize("degree", [9, 12, 13, 17, 24, 25, 31, 32])
+@pytest.mark.parametrize("values,P,R", [("pm1", 8, 16), ("pm1", 12, 10), ("fp32", 16, 16), ("bf16", 4, 9)])
+def test_long_lists_equal_per_step(sb, degree, values, P, R):
+    """Rows of 9 to 32 entries, in groups of 12 slots with remainders, on half and whole warps, several
+    passes a warp for the first shape.  (The generator's rows are of the degree or one off it; past 32
+    entries the per-step kernels serve.)"""
+    _, spec = regular(9000 if (values, P) == ("pm1", 8) else 1200, degree, degree)
+    if values == "pm1":
+        spec = _signs(spec)
+    prec = "auto" if values == "pm1" else values
+    kw = dict(precision=prec, gamma0=4.0 * P, eval_every=17)
+    a = _run(sb, spec, P, R, 40, 1, **kw)
+    b = _run(sb, spec, P, R, 40, 2, **kw)
+    longest = int(np.diff(spec[2]).max())
+    assert a[0].info().step_kernel == 0 and b[0].info().step_kernel == (4 if longest <= 32 else 0)
+    assert np.array_equal(a[1], b[1]) and np.array_equal(a[2], b[2])
+    for k in a[3]:
+        assert np.array_equal(a[3][k], b[3][k]), k
+
+
+@pytest.mark.parametrize("degree,variant,want", [(35, "threshold", 0), (9, "ballistic", 6)])
+def test_degrees_past_the_lists_stay_per_step(sb, degree, variant, want):
+    _, spec = regular(1200, degree, 5)
+    assert _run(sb, spec, 8, 16, 10, 2, variant=variant)[0].info().step_kernel == want
+
+
 @pytest.mark.parametrize("variant", ["threshold", "ballistic"])
 @pytest.mark.parametrize("cut", [1, 2, 3, 18])
 def test_stretches_and_restarts(sb, variant, cut):
