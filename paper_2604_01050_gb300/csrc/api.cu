@@ -228,7 +228,7 @@ sbqa_problem::~sbqa_problem() {
   if (tc_plan) tc_plan_free(tc_plan);
   if (tc4_plan) tc4_plan_free(tc4_plan);
   if (fx_plan) fx_plan_free(fx_plan);
-  d_fx_digits.release(true); d_fx_h.release(true);
+  d_fx_digits.release(true); d_fx_h.release(true); d_fx_spins.release(true);
   d_J8.release(true); d_FT.release(true); d_err.release(true);
   d_row_ptr.release(true); d_col.release(true); d_col_pm1.release(true); d_npos.release(true); d_val_f32.release(true);
   d_val_bf16.release(true); d_dense_f32.release(true); d_h.release(true); d_e_i32.release(true);
@@ -647,18 +647,18 @@ int prepare_tc_values(sbqa_problem *p) {
 // device.  Without the memory for them (or with row sums past the FP64 range)
 // the FP64 readout on the CUDA cores serves.
 int prepare_fx(sbqa_problem *p) {
-  if (p->fx_tried || !fx_eligible(p->Kp)) return SBQA_OK;
+  if (p->fx_tried || p->is_integer || !fx_eligible(p->n)) return SBQA_OK;
   p->fx_tried = true;
   DevBuf<unsigned long long> scratch;
-  if (p->d_fx_digits.alloc(fx_digit_bytes(p->Kp)) != cudaSuccess || p->d_fx_h.alloc(p->n) != cudaSuccess ||
+  if (p->d_fx_digits.alloc(fx_digit_bytes(p->n)) != cudaSuccess || p->d_fx_h.alloc(p->n) != cudaSuccess ||
       scratch.alloc(1) != cudaSuccess) {
     cudaGetLastError();
     p->d_fx_digits.release();
     p->d_fx_h.release();
     return SBQA_OK;
   }
-  const cudaError_t e = fx_plan_make(&p->fx_plan, p->d_e_f64.p, p->d_h_f64.p, p->n, p->Kp, p->d_fx_digits.p,
-                                     p->d_fx_h.p, scratch.p, nullptr);
+  const cudaError_t e = fx_plan_make(&p->fx_plan, p->d_e_f64.p, p->d_h_f64.p, p->n, p->d_fx_digits.p, p->d_fx_h.p,
+                                     scratch.p, nullptr);
   scratch.release(true);
   SBQA_CUDA(e);
   return SBQA_OK;
@@ -692,16 +692,16 @@ int prepare_dense_values(sbqa_problem *p, int precision) {
     }
     p->tc_op = op;
     // the readout runs on the tensor cores too when its energies are integers
-    // and the product is e4m3, and in fixed point when they are real and the
-    // operands bfloat16; otherwise on the CUDA cores (exact int64 or FP64)
+    // and the product is e4m3, and in fixed point when they are real; otherwise
+    // on the CUDA cores (exact int64, or FP64)
     int rc = prepare_tc_values(p);
     if (rc != SBQA_OK || (p->is_integer && op == kTcOpF8)) return rc;
     rc = upload_readout_values(p);
-    if (rc != SBQA_OK || p->is_integer || op == kTcOpF8) return rc;
-    return prepare_fx(p);
+    return rc != SBQA_OK ? rc : prepare_fx(p);
   }
   {
-    const int rc = upload_readout_values(p);
+    int rc = upload_readout_values(p);
+    if (rc == SBQA_OK) rc = prepare_fx(p);
     if (rc != SBQA_OK) return rc;
   }
   const int want = precision == SBQA_PREC_BF16 ? SBQA_PREC_BF16 : SBQA_PREC_FP32;
@@ -754,6 +754,10 @@ int memo_blocks(int (*query)()) {
 // The tensor-core kernels' shared-memory limits, set once per device (they last for the context).
 int tc_attributes_once() { return tc_set_attributes() == cudaSuccess ? 1 : 0; }
 
+// The spins of the fixed-point readout take the f buffer of the step before
+// where it holds bfloat16 operands.
+bool fx_spins_in_ft(const sbqa_problem *p) { return p->use_tc && p->tc_op != kTcOpF8; }
+
 int alloc_run(sbqa_problem *p, int S, int P, int R) {
   const int Ps = run_width(P);  // a run's columns: P replicas, then padding up to a power of two
   const int C = R * Ps;
@@ -786,6 +790,9 @@ int alloc_run(sbqa_problem *p, int S, int P, int R) {
   SBQA_CUDA(p->d_err.alloc(1));
   SBQA_CUDA(cudaMemsetAsync(p->d_err.p, 0, sizeof(int), p->stream));  // no trial launch reads a stale code
   p->S = S; p->P = P; p->R = R; p->C = C; p->Cp = Cp; p->Ps = Ps;
+  if (p->dense && p->fx_plan && !fx_spins_in_ft(p) &&
+      p->d_fx_spins.alloc(fx_spin_bytes(p->n, Cp) / sizeof(uint16_t)) != cudaSuccess)
+    cudaGetLastError();  // without them the FP64 readout serves
   if (p->use_tc) {
     SBQA_CUDA(p->d_FT.alloc(tc_ft_bytes(p->Kp, Cp, p->tc_op)));
     if (!p->tc_plan || p->tc_plan_ft != p->d_FT.p || p->tc_plan_cp != Cp || p->tc_plan_x != p->d_x.p ||
@@ -1305,8 +1312,10 @@ cudaError_t issue_readout(sbqa_problem *p, int step, cudaStream_t st) {
     e = launch_energy_csr(s, p->csr_readout(), E, p->best(), st);
   else if (tc && p->is_integer && p->tc_op == kTcOpF8)
     e = launch_energy_dense_tc(p->tc_plan, s, p->Kp, p->d_FT.p, step & 1, p->d_err.p, E, p->best(), st);
-  else if (tc && E.fx)
-    e = launch_energy_dense_fx(p->tc_plan, s, p->Kp, p->d_FT.p, step & 1, p->d_err.p, E, p->best(), st);
+  else if (E.fx && fx_spins_in_ft(p))
+    e = launch_energy_dense_fx(s, E, p->d_FT.p + size_t(step & 1) * s.Cp * p->Kp * 2, p->d_err.p, p->best(), st);
+  else if (E.fx && p->d_fx_spins.p)
+    e = launch_energy_dense_fx(s, E, p->d_fx_spins.p, p->d_err.p, p->best(), st);
   else
     e = launch_energy_dense(s, E, p->best(), st);
   if (e != cudaSuccess) return e;

@@ -14,7 +14,8 @@
 // are those of X and H and one of the result: an energy is closer to the
 // instance's than the FP64 sum in any order, whatever the order.
 // At N = 2000, R*P = 1024 the eight GEMMs (66 GFLOP, operands 64 MB, in L2)
-// and the kernels around them take 0.2 ms instead of 10.7.
+// and the kernels around them take 0.14 ms instead of 10.7; at N = 1000, R*P =
+// 256 the readout takes 0.04 ms instead of 1.34.
 #include <cmath>
 #include <cstdint>
 
@@ -28,7 +29,7 @@ constexpr int kFxMaxKp = 16384;  // 4.3 GB of digits; larger instances keep the 
 struct FxPlan {
   CUtensorMap A;  // digits [8 Kp][Kp] bfloat16, most significant plane first
   const int64_t *H;
-  int k;
+  int k, Kp;
 };
 
 // Largest row sum of |J_ij| + 2 |h_i| (bits of a non-negative double, which
@@ -63,9 +64,9 @@ __global__ void k_fx_digits(const double *J, const double *h, int N, int Kp, int
   if (j == 0 && i < N) H[i] = __double2ll_rn(scalbn(h[i], k));
 }
 
-// Spins S [N][Cp] (+1, -1; 0 past C) -> bfloat16 [Cp][Kp] in FT buffer b (zeros
-// for padded spins), through 64 x 64 tiles so that both sides are coalesced.
-__global__ void __launch_bounds__(256) k_sign_to_ft16(StateView s, uint16_t *FT, int Kp, int b) {
+// Spins S [N][Cp] (+1, -1; 0 past C) -> bfloat16 [Cp][Kp] (zeros for padded
+// spins), through 64 x 64 tiles so that both sides are coalesced.
+__global__ void __launch_bounds__(256) k_sign_to_ft16(StateView s, uint16_t *FT, int Kp) {
   __shared__ int8_t t[64][68];
   const int i0 = blockIdx.x * 64, c0 = blockIdx.y * 64;
   for (int q = threadIdx.x; q < 64 * 16; q += 256) {
@@ -79,7 +80,7 @@ __global__ void __launch_bounds__(256) k_sign_to_ft16(StateView s, uint16_t *FT,
     const int c = q >> 5, r = (q & 31) * 2;
     auto code = [](int8_t v) { return v == 0 ? 0u : (v > 0 ? 0x3F80u : 0xBF80u); };
     const uint32_t v = code(t[r][c]) | (code(t[r + 1][c]) << 16);
-    *reinterpret_cast<uint32_t *>(FT + (size_t(b) * s.Cp + c0 + c) * Kp + i0 + r) = v;
+    *reinterpret_cast<uint32_t *>(FT + size_t(c0 + c) * Kp + i0 + r) = v;
   }
 }
 
@@ -94,7 +95,7 @@ static_assert(kFxSmem <= 227 * 1024, "shared memory of one block");
 
 __global__ void __launch_bounds__(kFxThreads, 1)
     k_energy_dense_fx(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB, StateView s,
-                      int Kp, int b, int *err, const int64_t *H, int64_t *part) {
+                      int Kp, int *err, const int64_t *H, int64_t *part) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint8_t *sA = smem, *sB = smem + kFxStages * kTcTile;
@@ -132,7 +133,7 @@ __global__ void __launch_bounds__(kFxThreads, 1)
         if (use > 0 && !tc::mbar_wait(&empty[st], (use - 1) & 1, err, tc::ERR_WAIT_EMPTY)) break;
         tc::mbar_arrive_expect_tx(&full[st], 2 * kTcTile);
         tc::tma_load_2d(sA + st * kTcTile, &mapA, &full[st], kb * 64, d * Kp + m0);
-        tc::tma_load_2d(sB + st * kTcTile, &mapB, &full[st], kb * 64, b * s.Cp + n0);
+        tc::tma_load_2d(sB + st * kTcTile, &mapB, &full[st], kb * 64, n0);
       }
   } else if (warp == 17) {
     if (lane == 0) {
@@ -246,11 +247,16 @@ __global__ void k_energy_fx_final(int C, int Cp, int blocks, int k, const int64_
   }
 }
 
-size_t fx_digit_bytes(int Kp) { return size_t(kFxDigits) * Kp * Kp * 2; }
-bool fx_eligible(int Kp) { return Kp <= kFxMaxKp; }
+static int tc_padded(int N) { return (N + 127) / 128 * 128; }
+size_t fx_digit_bytes(int N) { return size_t(kFxDigits) * tc_padded(N) * tc_padded(N) * 2; }
+size_t fx_spin_bytes(int N, int Cp) { return size_t(Cp) * tc_padded(N) * 2; }
+// From N = 64 on: below, the FP64 sums are short, and the partial sums and the
+// spins would not fit the buffers they are given.
+bool fx_eligible(int N) { return N >= 64 && tc_padded(N) <= kFxMaxKp; }
 
-cudaError_t fx_plan_make(void **plan, const double *J, const double *h, int N, int Kp, void *digits, int64_t *H,
+cudaError_t fx_plan_make(void **plan, const double *J, const double *h, int N, void *digits, int64_t *H,
                          unsigned long long *scratch, cudaStream_t st) {
+  const int Kp = tc_padded(N);
   *plan = nullptr;
   cudaError_t e = cudaFuncSetAttribute((const void *)k_energy_dense_fx, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        kFxSmem);
@@ -266,6 +272,7 @@ cudaError_t fx_plan_make(void **plan, const double *J, const double *h, int N, i
   auto *p = new FxPlan();
   p->k = most > 0.0 ? 61 - std::ilogb(most) : 0;  // row sums below 2^62 after scaling
   p->H = H;
+  p->Kp = Kp;
   const size_t total = size_t(Kp) * Kp;
   k_fx_digits<<<unsigned((total + 255) / 256), 256, 0, st>>>(J, h, N, Kp, p->k, static_cast<uint16_t *>(digits), H);
   e = cudaGetLastError();
@@ -283,18 +290,21 @@ cudaError_t fx_plan_make(void **plan, const double *J, const double *h, int N, i
 
 void fx_plan_free(void *plan) { delete static_cast<FxPlan *>(plan); }
 
-cudaError_t launch_energy_partials_fx(const void *tc_plan, const void *fx_plan, const StateView &s, int Kp,
-                                      uint8_t *FT, int b, int *err, const BestView &best, cudaStream_t st) {
+cudaError_t launch_energy_partials_fx(const void *fx_plan, const StateView &s, void *spins, int *err,
+                                      const BestView &best, cudaStream_t st) {
   const auto *p = static_cast<const FxPlan *>(fx_plan);
-  k_sign_to_ft16<<<dim3(unsigned(Kp / 64), unsigned(s.Cp / 64)), 256, 0, st>>>(s, reinterpret_cast<uint16_t *>(FT), Kp,
-                                                                             b);
+  const int Kp = p->Kp;
+  CUtensorMap B;
+  if (!tc_make_map(&B, spins, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, uint64_t(s.Cp), uint64_t(Kp), 64, 128,
+                   CU_TENSOR_MAP_SWIZZLE_128B))
+    return cudaErrorInvalidValue;
+  k_sign_to_ft16<<<dim3(unsigned(Kp / 64), unsigned(s.Cp / 64)), 256, 0, st>>>(s, static_cast<uint16_t *>(spins), Kp);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   const dim3 grid(unsigned(s.Cp / kTcBN), unsigned(Kp / kTcBM));
   // the partial sums of 128 rows take 16 bytes, those of the FP64 kernel's 32 rows 8
   int64_t *part = reinterpret_cast<int64_t *>(best.part_f64);
-  k_energy_dense_fx<<<grid, kFxThreads, kFxSmem, st>>>(p->A, static_cast<const TcMaps *>(tc_plan)->B, s, Kp, b, err,
-                                                       p->H, part);
+  k_energy_dense_fx<<<grid, kFxThreads, kFxSmem, st>>>(p->A, B, s, Kp, err, p->H, part);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   k_energy_fx_final<<<unsigned((s.C + 7) / 8), 256, 0, st>>>(s.C, s.Cp, Kp / kTcBM, p->k, part, best.e_f64);
   return cudaGetLastError();

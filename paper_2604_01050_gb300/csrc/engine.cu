@@ -334,14 +334,16 @@ int readout(sbqa_engine *e, Request &r, cudaStream_t st) {
   sbqa_problem *p = r.prob;
   const StateView s = r.state_view();
   const EnergyView ev = problem_energy_view(p);
-  // as sbqa_run reads out: integer energies (J and h) of e4m3 products and real ones of bfloat16
-  // products on the tensor cores, others on the CUDA cores
+  // as sbqa_run reads out: integer energies (J and h) of e4m3 products and real ones on the tensor
+  // cores, others on the CUDA cores; the request's last readout leaves its momenta unused, so the
+  // spins of the real ones take their place
   const bool tc8 = p->dense && r.tc_plan && p->is_integer && p->tc_op == kTcOpF8;
-  const bool fx = p->dense && r.tc_plan && ev.fx && tc_op_of(r.tc_plan) != kTcOpF8, tc = tc8 || fx;
-  cudaError_t err = tc8 ? launch_energy_dense_tc(r.tc_plan, s, p->Kp, r.FT, (r.S - 1) & 1, r.err, ev, r.best_view(), st)
-                    : fx ? launch_energy_dense_fx(r.tc_plan, s, p->Kp, r.FT, (r.S - 1) & 1, r.err, ev, r.best_view(), st)
-                       : p->dense ? launch_energy_dense(s, ev, r.best_view(), st)
-                                  : launch_energy_csr(s, problem_csr_readout_view(p), ev, r.best_view(), st);
+  const bool fx = p->dense && ev.fx, tc = tc8 || fx;
+  cudaError_t err;
+  if (tc8) err = launch_energy_dense_tc(r.tc_plan, s, p->Kp, r.FT, (r.S - 1) & 1, r.err, ev, r.best_view(), st);
+  else if (fx) err = launch_energy_dense_fx(s, ev, r.y, r.err, r.best_view(), st);
+  else if (p->dense) err = launch_energy_dense(s, ev, r.best_view(), st);
+  else err = launch_energy_csr(s, problem_csr_readout_view(p), ev, r.best_view(), st);
   if (err == cudaSuccess) err = launch_best(s, ev, r.best_view(), r.S - 1, st);
   e->kernels_launched += tc ? 5 : 4;  // signs, (sign codes,) energies, their final sums, best
   if (err != cudaSuccess) return set_error(SBQA_ERR_CUDA, std::string("engine readout: ") + cudaGetErrorString(err));

@@ -309,10 +309,10 @@ cudaError_t launch_energy_dense_tc(const void *plan, const StateView &s, int Kp,
   return launch_final(s, E, b, st);
 }
 
-cudaError_t launch_energy_dense_fx(const void *plan, const StateView &s, int Kp, uint8_t *FT, int buffer, int *err,
-                                   const EnergyView &E, const BestView &b, cudaStream_t st) {
+cudaError_t launch_energy_dense_fx(const StateView &s, const EnergyView &E, void *spins, int *err, const BestView &b,
+                                   cudaStream_t st) {
   const cudaError_t e = launch_sign(s, st);
-  return e != cudaSuccess ? e : launch_energy_partials_fx(plan, E.fx, s, Kp, FT, buffer, err, b, st);
+  return e != cudaSuccess ? e : launch_energy_partials_fx(E.fx, s, spins, err, b, st);
 }
 
 // ---------------------------------------------------------------- best per run

@@ -87,7 +87,7 @@ struct EnergyView {
   const int32_t *val_i32;  // [nnz] or [N][N], integer instances
   const double *h_f64;     // [N]
   const int64_t *h_i64;    // [N]
-  const void *fx;          // fixed-point plan of a real dense instance on the tensor cores, or null (energy_fixed.cu)
+  const void *fx;          // fixed-point plan of a real dense instance, or null (energy_fixed.cu)
 };
 
 struct BestView {
@@ -364,20 +364,21 @@ cudaError_t launch_energy_partials_tc(const void *plan, const StateView &s, int 
                                       const int64_t *h_i64, int64_t *part, int nblk, cudaStream_t st);
 cudaError_t launch_energy_dense_tc(const void *plan, const StateView &s, int Kp, uint8_t *FT, int buffer, int *err,
                                    const EnergyView &E, const BestView &b, cudaStream_t st);
-// Readout energies of a real dense instance whose operands are bfloat16: J and
-// h in 64-bit fixed point, one bfloat16 operand per byte (energy_fixed.cu).
-// The plan is made once per problem from the FP64 J [N][N] and h [N] into
-// digits (fx_digit_bytes) and H [N]; *plan stays null when the row sums leave
-// the FP64 range.  The spins take FT buffer b, as above.
-bool fx_eligible(int Kp);
-size_t fx_digit_bytes(int Kp);
-cudaError_t fx_plan_make(void **plan, const double *J, const double *h, int N, int Kp, void *digits, int64_t *H,
+// Readout energies of a real dense instance on the tensor cores: J and h in
+// 64-bit fixed point, one bfloat16 operand per byte (energy_fixed.cu).  The
+// plan is made once per problem from the FP64 J [N][N] and h [N] into digits
+// (fx_digit_bytes) and H [N]; *plan stays null when the row sums leave the
+// FP64 range.  The spins take fx_spin_bytes at `spins` (16-byte aligned).
+bool fx_eligible(int N);
+size_t fx_digit_bytes(int N);
+size_t fx_spin_bytes(int N, int Cp);
+cudaError_t fx_plan_make(void **plan, const double *J, const double *h, int N, void *digits, int64_t *H,
                          unsigned long long *scratch, cudaStream_t st);
 void fx_plan_free(void *plan);
-cudaError_t launch_energy_partials_fx(const void *tc_plan, const void *fx_plan, const StateView &s, int Kp,
-                                      uint8_t *FT, int b, int *err, const BestView &best, cudaStream_t st);
-cudaError_t launch_energy_dense_fx(const void *plan, const StateView &s, int Kp, uint8_t *FT, int buffer, int *err,
-                                   const EnergyView &E, const BestView &b, cudaStream_t st);
+cudaError_t launch_energy_partials_fx(const void *fx_plan, const StateView &s, void *spins, int *err,
+                                      const BestView &best, cudaStream_t st);
+cudaError_t launch_energy_dense_fx(const StateView &s, const EnergyView &E, void *spins, int *err, const BestView &b,
+                                   cudaStream_t st);
 // sign(x) into Sg, energies of every column into b.e_int / b.e_f64.
 cudaError_t launch_energy_csr(const StateView &s, const CsrView &J, const EnergyView &E,
                               const BestView &b, cudaStream_t st);

@@ -165,11 +165,12 @@ struct sbqa_problem {
   sbqa::DevBuf<double> d_e_f64;
   sbqa::DevBuf<int64_t> d_h_i64;
   sbqa::DevBuf<double> d_h_f64;
-  // fixed-point readout of a real J on the tensor cores (energy_fixed.cu); made once
+  // fixed-point readout of a real dense J (energy_fixed.cu); made once
   sbqa::DevBuf<uint8_t> d_fx_digits;
   sbqa::DevBuf<int64_t> d_fx_h;
   void *fx_plan = nullptr;
   bool fx_tried = false;
+  sbqa::DevBuf<uint16_t> d_fx_spins;  // its spins, where no f buffer of the tensor cores takes them
 
   // schedule
   bool have_params = false;
@@ -335,7 +336,7 @@ struct sbqa_problem {
     EnergyView e;
     e.is_integer = is_integer ? 1 : 0;
     e.val_i32 = d_e_i32.p; e.val_f64 = d_e_f64.p; e.h_i64 = d_h_i64.p; e.h_f64 = d_h_f64.p;
-    e.fx = use_tc && tc_op != sbqa::kTcOpF8 ? fx_plan : nullptr;
+    e.fx = fx_plan;
     return e;
   }
   BestView best() const {

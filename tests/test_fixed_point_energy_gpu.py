@@ -32,13 +32,15 @@ def _instance(kind, n, rng):
     return up + up.T, h
 
 
-@pytest.mark.parametrize("n,P,R", [(256, 1, 3), (257, 8, 17), (383, 5, 40), (640, 16, 16)])
+@pytest.mark.parametrize("prec", ["bf16", "fp32"])
+@pytest.mark.parametrize("n,P,R", [(64, 4, 33), (65, 2, 70), (129, 7, 3), (256, 1, 3), (257, 8, 17), (383, 5, 40),
+                                   (640, 16, 16)])
 @pytest.mark.parametrize("kind", ["gauss", "tail", "tiny", "huge", "field"])
-def test_energies_are_rounded_once(sb, n, P, R, kind):
+def test_energies_are_rounded_once(sb, n, P, R, kind, prec):
     rng = np.random.default_rng(n)
     J, h = _instance(kind, n, rng)
     pb = sb.create_problem_dense(J, h)
-    sb.set_schedule(pb, precision="bf16", gamma0=4.0 * P)
+    sb.set_schedule(pb, precision=prec, gamma0=4.0 * P)
     sb.run(pb, 30, P, R, seed=4)
     e, _ = sb.get_energies(pb)
     x, _, _ = sb.get_state(pb)
@@ -52,6 +54,39 @@ def test_energies_are_rounded_once(sb, n, P, R, kind):
         exact = -math.fsum(np.concatenate([J[iu] * s[iu[0]] * s[iu[1]], h * s]))
         tol = unit * 0.5 * (n * n / 2 + n) + 2.0 ** -52 * abs(exact)
         assert abs(e[r, k] - exact) <= tol, (e[r, k], exact)
+
+
+@pytest.mark.parametrize("n,prec", [(200, "fp32"), (300, "fp32"), (300, "bf16")])
+def test_engine_and_solve_read_out_alike(sb, n, prec):
+    rng = np.random.default_rng(n)
+    J, h = _instance("gauss", n, rng)
+    pb = sb.create_problem_dense(J, h)
+    sb.set_schedule(pb, precision=prec, gamma0=32.0)
+    eng = sb.engine_create(64 << 20, 4, 7)
+    rid = sb.engine_submit(eng, pb, 40, 8, 5, seed=9)
+    while rid not in sb.engine_step(eng):
+        pass
+    a = sb.engine_result(eng, rid)
+    sb.run(pb, 40, 8, 5, seed=9)
+    b = sb.get_best(pb)
+    for k in a:
+        assert np.array_equal(a[k], b[k]), k
+
+
+def test_integer_couplings_beside_a_real_field(sb):
+    """The e4m3 product keeps its f buffers; the spins of the readout have a buffer of their own."""
+    rng = np.random.default_rng(2)
+    up = np.triu(rng.integers(-3, 4, (300, 300)).astype(float), 1)
+    J, h = up + up.T, rng.standard_normal(300)
+    pb = sb.create_problem_dense(J, h)
+    sb.set_schedule(pb, gamma0=32.0, eval_every=6)
+    sb.run(pb, 31, 8, 5, seed=9)
+    assert pb.info().step_kernel in (2, 5, 8, 9, 15, 16)
+    e, _ = sb.get_energies(pb)
+    x, _, _ = sb.get_state(pb)
+    s = np.where(x >= 0, 1.0, -1.0)
+    ref = -0.5 * np.einsum("rki,ij,rkj->rk", s, J, s) - s @ h
+    assert np.allclose(e, ref, rtol=1e-12, atol=0)
 
 
 def test_row_sums_past_the_fp64_range(sb):
