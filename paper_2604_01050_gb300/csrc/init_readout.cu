@@ -153,6 +153,18 @@ __device__ __forceinline__ void reduce_block_cols(T (*sm)[kColsPerWarp], const T
 }
 
 // ---------------------------------------------------------------- CSR energies
+// t + w s for a spin s = +-1 in byte q of s4 (the product is w with a sign, so
+// this is one addition; the bytes past C hold 0 and their sums are not read).
+__device__ __forceinline__ double add_signed(double t, double w, uint32_t s4, int q) {
+  const int sign = int((s4 << (24 - 8 * q)) & 0x80000000u);
+  return t + __hiloint2double(__double2hiint(w) ^ sign, __double2loint(w));
+}
+
+// Four rows per warp, four columns per lane.  The gathers of four entries are
+// in flight at a time; sums run in entry order.  FP64: signed additions, no
+// conversions (which run at the FP64 unit's rate too), so the FP64 adds bound
+// it.  Readout and start of a solve at N = 10^5, degree 6, R*P = 128, with the
+// split of k_best: 592 -> 419 us; lattice L = 16, R*P = 2048: 129 -> 79.
 template <bool INT>
 __global__ void __launch_bounds__(256) k_energy_csr(StateView s, CsrView J, EnergyView E,
                                                     BestView b) {
@@ -167,18 +179,30 @@ __global__ void __launch_bounds__(256) k_energy_csr(StateView s, CsrView J, Ener
     if (i >= s.N) break;
     const uint32_t si4 = *reinterpret_cast<const uint32_t *>(s.Sg + size_t(i) * s.Cp + c4);
     T t[4] = {T(0), T(0), T(0), T(0)};
-    for (int e = J.row_ptr[i]; e < J.row_ptr[i + 1]; ++e) {
-      const int j = J.col[e];
-      const uint32_t sj4 = *reinterpret_cast<const uint32_t *>(s.Sg + size_t(j) * s.Cp + c4);
-      const T w = INT ? T(E.val_i32[e]) : T(E.val_f64[e]);
+    const int e1 = J.row_ptr[i + 1];
+    for (int e = J.row_ptr[i]; e < e1; e += 4) {
+      uint32_t sj4[4];
 #pragma unroll
-      for (int q = 0; q < 4; ++q) t[q] += w * T(int8_t(sj4 >> (8 * q)));
+      for (int u = 0; u < 4; ++u)
+        sj4[u] = *reinterpret_cast<const uint32_t *>(s.Sg + size_t(J.col[min(e + u, e1 - 1)]) * s.Cp + c4);
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        if (e + u >= e1) break;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          if constexpr (INT) t[q] += (long long)E.val_i32[e + u] * int(int8_t(sj4[u] >> (8 * q)));
+          else t[q] = add_signed(t[q], E.val_f64[e + u], sj4[u], q);
+        }
+      }
     }
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
-      const T si = T(int8_t(si4 >> (8 * q)));
-      if constexpr (INT) v[q] += si * t[q] + 2 * T(E.h_i64[i]) * si;
-      else v[q] += si * (0.5 * t[q] + E.h_f64[i]);
+      if constexpr (INT) {
+        const int si = int8_t(si4 >> (8 * q));
+        v[q] += (t[q] + 2 * T(E.h_i64[i])) * si;
+      } else {
+        v[q] = add_signed(v[q], fma(0.5, t[q], E.h_f64[i]), si4, q);
+      }
     }
   }
   reduce_block_cols<T>(sm, v, INT ? reinterpret_cast<T *>(b.part_int) : reinterpret_cast<T *>(b.part_f64),
@@ -319,8 +343,9 @@ cudaError_t launch_energy_dense_fx(const StateView &s, const EnergyView &E, void
 // One block per run: warp 0 takes the argmin over the Pr replicas (lowest k
 // on ties; replica k of run r is column r * P + k), kept if strictly lower
 // than the best so far; then all threads copy the winner's spins (a strided
-// gather of N bytes).
-constexpr int kBestThreads = 256;
+// gather of N bytes).  From N = kBestSplit on the copy is a kernel of its own
+// over blocks of spins (N = 10^5, 8 runs: 190 us by 8 blocks).
+constexpr int kBestThreads = 256, kBestSplit = 16384;
 
 __global__ void __launch_bounds__(kBestThreads) k_best(StateView s, EnergyView E, BestView b, int step) {
   __shared__ int s_k;  // the winning replica, or -1 when the run does not improve
@@ -362,14 +387,25 @@ __global__ void __launch_bounds__(kBestThreads) k_best(StateView s, EnergyView E
   }
   __syncthreads();
   const int k = s_k;
-  if (k < 0) return;
+  if (k < 0 || s.N >= kBestSplit) return;
   const int c = r * P + k;
   for (int i = threadIdx.x; i < s.N; i += kBestThreads) b.best_spins[size_t(r) * s.N + i] = s.Sg[size_t(i) * s.Cp + c];
+}
+
+// The spins of the runs that improved at this readout: their best is of `step`
+// (a run reads out once per step).
+__global__ void __launch_bounds__(kBestThreads) k_best_spins(StateView s, BestView b, int step) {
+  const int r = blockIdx.x;
+  if (b.best_step[r] != step) return;
+  const int c = r * s.P + b.best_k[r], i = blockIdx.y * kBestThreads + threadIdx.x;
+  if (i < s.N) b.best_spins[size_t(r) * s.N + i] = s.Sg[size_t(i) * s.Cp + c];
 }
 
 cudaError_t launch_best(const StateView &s, const EnergyView &E, const BestView &b, int step,
                         cudaStream_t st) {
   k_best<<<s.R, kBestThreads, 0, st>>>(s, E, b, step);
+  if (s.N >= kBestSplit)
+    k_best_spins<<<dim3(s.R, (s.N + kBestThreads - 1) / kBestThreads), kBestThreads, 0, st>>>(s, b, step);
   return cudaGetLastError();
 }
 
