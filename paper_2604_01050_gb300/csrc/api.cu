@@ -229,16 +229,14 @@ sbqa_problem::~sbqa_problem() {
   if (tc4_plan) tc4_plan_free(tc4_plan);
   if (fx_plan) fx_plan_free(fx_plan);
   d_fx_digits.release(true); d_fx_h.release(true); d_fx_spins.release(true);
-  d_J8.release(true); d_FT.release(true); d_err.release(true);
+  d_J8.release(true); d_FT.release(true); d_results.release(true);
   d_row_ptr.release(true); d_col.release(true); d_col_pm1.release(true); d_npos.release(true); d_val_f32.release(true);
   d_val_bf16.release(true); d_dense_f32.release(true); d_h.release(true); d_e_i32.release(true);
   d_e_f64.release(true); d_h_i64.release(true); d_h_f64.release(true); d_x.release(true); d_y.release(true);
   d_jcopy_i8.release(true);
   d_F0.release(true); d_F1.release(true); d_Fx0.release(true); d_Fx1.release(true); d_Sg.release(true);
   d_ell_col.release(true); d_ell_meta.release(true); d_ell_val.release(true); d_ka.release(true); d_dl.release(true);
-  d_kj.release(true); d_ei.release(true); d_part_i.release(true); d_best_ei.release(true); d_ef.release(true);
-  d_part_f.release(true); d_best_e.release(true); d_best_k.release(true); d_best_step.release(true);
-  d_have.release(true); d_best_spins.release(true); d_bar.release(true); d_tc_flags.release(true);
+  d_kj.release(true); d_part_i.release(true); d_part_f.release(true); d_have.release(true); d_bar.release(true); d_tc_flags.release(true);
   d_J4.release(true); d_FT4.release(true);
 }
 
@@ -758,6 +756,38 @@ int tc_attributes_once() { return tc_set_attributes() == cudaSuccess ? 1 : 0; }
 // where it holds bfloat16 operands.
 bool fx_spins_in_ft(const sbqa_problem *p) { return p->use_tc && p->tc_op != kTcOpF8; }
 
+// Offsets of the parts of a run's results (each 16-byte aligned).
+struct ResultLayout {
+  size_t best_e, best_ei, best_k, best_step, ef, ei, spins, end;
+  ResultLayout(size_t n, size_t R, size_t Cp) {
+    auto up = [](size_t b) { return (b + 15) / 16 * 16; };
+    best_e = 16;  // behind the error flag
+    best_ei = best_e + up(8 * R);
+    best_k = best_ei + up(8 * R);
+    best_step = best_k + up(4 * R);
+    ef = best_step + up(4 * R);
+    ei = ef + 8 * Cp;
+    spins = ei + 8 * Cp;
+    end = spins + R * n;
+  }
+};
+
+cudaError_t carve_results(sbqa_problem *p, int R, int Cp) {
+  const ResultLayout l(size_t(p->n), size_t(R), size_t(Cp));
+  const cudaError_t e = p->d_results.alloc(l.end);
+  if (e != cudaSuccess) return e;
+  uint8_t *b = p->d_results.p;
+  p->d_err.p = reinterpret_cast<int *>(b);
+  p->d_best_e.p = reinterpret_cast<double *>(b + l.best_e);
+  p->d_best_ei.p = reinterpret_cast<int64_t *>(b + l.best_ei);
+  p->d_best_k.p = reinterpret_cast<int32_t *>(b + l.best_k);
+  p->d_best_step.p = reinterpret_cast<int32_t *>(b + l.best_step);
+  p->d_ef.p = reinterpret_cast<double *>(b + l.ef);
+  p->d_ei.p = reinterpret_cast<int64_t *>(b + l.ei);
+  p->d_best_spins.p = reinterpret_cast<int8_t *>(b + l.spins);
+  return cudaSuccess;
+}
+
 int alloc_run(sbqa_problem *p, int S, int P, int R) {
   const int Ps = run_width(P);  // a run's columns: P replicas, then padding up to a power of two
   const int C = R * Ps;
@@ -776,18 +806,11 @@ int alloc_run(sbqa_problem *p, int S, int P, int R) {
   SBQA_CUDA(p->d_ka.alloc(size_t(std::max(S, 1))));
   SBQA_CUDA(p->d_dl.alloc(size_t(S) + 1));
   SBQA_CUDA(p->d_kj.alloc(size_t(std::max(S, 1)) * R));
-  SBQA_CUDA(p->d_ei.alloc(Cp));
-  SBQA_CUDA(p->d_ef.alloc(Cp));
   const size_t parts = size_t(energy_row_blocks(p->n)) * Cp;
   if (p->is_integer) SBQA_CUDA(p->d_part_i.alloc(parts));
   else SBQA_CUDA(p->d_part_f.alloc(parts));
-  SBQA_CUDA(p->d_best_ei.alloc(R));
-  SBQA_CUDA(p->d_best_e.alloc(R));
-  SBQA_CUDA(p->d_best_k.alloc(R));
-  SBQA_CUDA(p->d_best_step.alloc(R));
   SBQA_CUDA(p->d_have.alloc(R));
-  SBQA_CUDA(p->d_best_spins.alloc(size_t(R) * p->n));
-  SBQA_CUDA(p->d_err.alloc(1));
+  SBQA_CUDA(carve_results(p, R, Cp));
   SBQA_CUDA(cudaMemsetAsync(p->d_err.p, 0, sizeof(int), p->stream));  // no trial launch reads a stale code
   p->S = S; p->P = P; p->R = R; p->C = C; p->Cp = Cp; p->Ps = Ps;
   if (p->dense && p->fx_plan && !fx_spins_in_ft(p) &&
@@ -1536,6 +1559,19 @@ DenseView sbqa::problem_dense_view(const sbqa_problem *p) {
   return d;
 }
 
+// Waits for the handle's work and copies the first `bytes` of its results: one
+// copy of the error flag and whatever else the caller wants.
+static int fetch_results(sbqa_problem *p, size_t bytes, std::vector<uint8_t> *buf) {
+  buf->resize(bytes);
+  SBQA_CUDA(p->stream ? cudaStreamSynchronize(p->stream) : cudaDeviceSynchronize());
+  SBQA_CUDA(cudaGetLastError());
+  SBQA_CUDA(cudaMemcpy(buf->data(), p->d_results.p, bytes, cudaMemcpyDeviceToHost));
+  int err = 0;
+  std::memcpy(&err, buf->data(), sizeof(err));
+  if (err != 0) return fail(SBQA_ERR_TIMEOUT, "a bounded device wait gave up (code " + std::to_string(err) + ")");
+  return SBQA_OK;
+}
+
 extern "C" {
 
 int sbqa_version(void) { return 100; }
@@ -1942,7 +1978,7 @@ int sbqa_run(sbqa_problem *p, int32_t steps, int32_t P, int32_t R, uint64_t seed
   }
   sbqa_problem::Key key;
   key.S = steps; key.P = P; key.R = R; key.eval = p->prm.eval_every; key.kind = p->kind;
-  key.dense = p->dense ? 1 : 0; key.x = p->d_x.p; key.kj = p->d_kj.p;
+  key.dense = p->dense ? 1 : 0; key.x = p->d_x.p; key.kj = p->d_kj.p; key.results = p->d_results.p;
   key.kc = p->tables.kc; key.kx = p->tables.kx; key.tc = p->use_tc ? 1 + p->tc_op : 0; key.variant = p->csr_variant;
   key.fvar = p->prm.variant;
   if (!(p->graph && p->graph_key == key)) {
@@ -1980,9 +2016,8 @@ int sbqa_synchronize(sbqa_problem *p) {
   SBQA_CUDA(p->stream ? cudaStreamSynchronize(p->stream) : cudaDeviceSynchronize());
   SBQA_CUDA(cudaGetLastError());
   if (p->d_err.p) {
-    int err = 0;
-    SBQA_CUDA(cudaMemcpy(&err, p->d_err.p, sizeof(int), cudaMemcpyDeviceToHost));
-    if (err != 0) return fail(SBQA_ERR_TIMEOUT, "a bounded device wait gave up (code " + std::to_string(err) + ")");
+    std::vector<uint8_t> buf;
+    return fetch_results(p, sizeof(int), &buf);
   }
   return SBQA_OK;
 }
@@ -1991,36 +2026,39 @@ int sbqa_get_best(sbqa_problem *p, int8_t *spins, double *energy, int64_t *energ
                   int32_t *step) {
   if (!p) return fail(SBQA_ERR_INVALID_ARG, "null problem");
   if (!p->finished) return fail(SBQA_ERR_STATE, "no finished readout");
-  int rc = sbqa_synchronize(p);
-  if (rc != SBQA_OK) return rc;
   DeviceGuard g(p->device);
-  const int R = p->R;
-  if (spins) SBQA_CUDA(cudaMemcpy(spins, p->d_best_spins.p, size_t(R) * p->n, cudaMemcpyDeviceToHost));
-  if (energy) SBQA_CUDA(cudaMemcpy(energy, p->d_best_e.p, R * sizeof(double), cudaMemcpyDeviceToHost));
-  if (energy_int && p->is_integer)
-    SBQA_CUDA(cudaMemcpy(energy_int, p->d_best_ei.p, R * sizeof(int64_t), cudaMemcpyDeviceToHost));
-  if (replica) SBQA_CUDA(cudaMemcpy(replica, p->d_best_k.p, R * sizeof(int32_t), cudaMemcpyDeviceToHost));
-  if (step) SBQA_CUDA(cudaMemcpy(step, p->d_best_step.p, R * sizeof(int32_t), cudaMemcpyDeviceToHost));
+  const size_t R = size_t(p->R), n = size_t(p->n);
+  const ResultLayout l(n, R, size_t(p->Cp));
+  // the spins come with the rest where they are few, else straight to the caller
+  const bool together = spins && R * n <= (size_t(64) << 10) && l.ef + 2 * 8 * size_t(p->Cp) <= (size_t(128) << 10);
+  std::vector<uint8_t> buf;
+  const int rc = fetch_results(p, together ? l.end : l.ef, &buf);
+  if (rc != SBQA_OK) return rc;
+  if (together) std::memcpy(spins, buf.data() + l.spins, R * n);
+  else if (spins) SBQA_CUDA(cudaMemcpy(spins, p->d_best_spins.p, R * n, cudaMemcpyDeviceToHost));
+  if (energy) std::memcpy(energy, buf.data() + l.best_e, R * sizeof(double));
+  if (energy_int && p->is_integer) std::memcpy(energy_int, buf.data() + l.best_ei, R * sizeof(int64_t));
+  if (replica) std::memcpy(replica, buf.data() + l.best_k, R * sizeof(int32_t));
+  if (step) std::memcpy(step, buf.data() + l.best_step, R * sizeof(int32_t));
   return SBQA_OK;
 }
 
 int sbqa_get_energies(sbqa_problem *p, double *energy, int64_t *energy_int) {
   if (!p) return fail(SBQA_ERR_INVALID_ARG, "null problem");
   if (!p->finished) return fail(SBQA_ERR_STATE, "no finished readout");
-  int rc = sbqa_synchronize(p);
-  if (rc != SBQA_OK) return rc;
   DeviceGuard g(p->device);
+  const ResultLayout l(size_t(p->n), size_t(p->R), size_t(p->Cp));
+  std::vector<uint8_t> buf;
+  const int rc = fetch_results(p, l.spins, &buf);
+  if (rc != SBQA_OK) return rc;
   // device energies by column r * Ps + k; the caller gets [r][k] for k < P
-  auto gather = [&](auto *out, const auto *dev) -> int {
+  auto gather = [&](auto *out, size_t off) {
     using T = std::remove_pointer_t<decltype(out)>;
-    std::vector<T> buf(size_t(p->C));
-    SBQA_CUDA(cudaMemcpy(buf.data(), dev, size_t(p->C) * sizeof(T), cudaMemcpyDeviceToHost));
-    for (int r = 0; r < p->R; ++r)
-      for (int k = 0; k < p->P; ++k) out[size_t(r) * p->P + k] = buf[size_t(r) * p->Ps + k];
-    return SBQA_OK;
+    const T *in = reinterpret_cast<const T *>(buf.data() + off);
+    for (int r = 0; r < p->R; ++r) std::memcpy(out + size_t(r) * p->P, in + size_t(r) * p->Ps, p->P * sizeof(T));
   };
-  if (energy && (rc = gather(energy, p->d_ef.p)) != SBQA_OK) return rc;
-  if (energy_int && p->is_integer && (rc = gather(energy_int, p->d_ei.p)) != SBQA_OK) return rc;
+  if (energy) gather(energy, l.ef);
+  if (energy_int && p->is_integer) gather(energy_int, l.ei);
   return SBQA_OK;
 }
 

@@ -100,6 +100,12 @@ struct DevBuf {
   }
 };
 
+// A part of a DevBuf that another member owns.
+template <typename T>
+struct DevView {
+  T *p = nullptr;
+};
+
 }  // namespace sbqa
 
 using sbqa::BestView;
@@ -158,7 +164,14 @@ struct sbqa_problem {
   const void *tc_plan_ft = nullptr;  // FT buffer the plan was made for
   const void *tc_plan_x = nullptr;   // state buffer the plan was made for
   int tc_plan_cp = 0;
-  sbqa::DevBuf<int> d_err;
+  // what a run reports, in one block (carve_results, api.cu) so that one copy fetches it:
+  // error flag, best energies, replicas and steps, energies of all columns, best spins
+  sbqa::DevBuf<uint8_t> d_results;
+  sbqa::DevView<int> d_err;
+  sbqa::DevView<double> d_best_e, d_ef;
+  sbqa::DevView<int64_t> d_best_ei, d_ei;
+  sbqa::DevView<int32_t> d_best_k, d_best_step;
+  sbqa::DevView<int8_t> d_best_spins;
   sbqa::DevBuf<float> d_h;
   // device: readout operands
   sbqa::DevBuf<int32_t> d_e_i32;
@@ -234,10 +247,9 @@ struct sbqa_problem {
   sbqa::DevBuf<float> d_Fx0, d_Fx1;  // f(x) = x buffers of the ballistic form
   sbqa::DevBuf<int8_t> d_Sg;
   sbqa::DevBuf<float> d_ka, d_dl, d_kj;
-  sbqa::DevBuf<int64_t> d_ei, d_part_i, d_best_ei;
-  sbqa::DevBuf<double> d_ef, d_part_f, d_best_e;
-  sbqa::DevBuf<int32_t> d_best_k, d_best_step, d_have;
-  sbqa::DevBuf<int8_t> d_best_spins;
+  sbqa::DevBuf<int64_t> d_part_i;
+  sbqa::DevBuf<double> d_part_f;
+  sbqa::DevBuf<int32_t> d_have;
   StepTables tables{};
 
   // cached graph of the step loop + readouts of a full run
@@ -246,9 +258,9 @@ struct sbqa_problem {
   struct Key {
     int S = -1, P = -1, R = -1, eval = -1, kind = -1, dense = -1, tc = -1, variant = -1, fvar = -1;
     float kc = 0.f, kx = 0.f;  // step constants are kernel arguments in the graph
-    const void *x = nullptr, *kj = nullptr;
+    const void *x = nullptr, *kj = nullptr, *results = nullptr;
     bool operator==(const Key &o) const {
-      return S == o.S && P == o.P && R == o.R && eval == o.eval && kind == o.kind &&
+      return S == o.S && P == o.P && R == o.R && results == o.results && eval == o.eval && kind == o.kind &&
              dense == o.dense && tc == o.tc && variant == o.variant && fvar == o.fvar && x == o.x && kj == o.kj &&
              std::memcmp(&kc, &o.kc, sizeof(float)) == 0 && std::memcmp(&kx, &o.kx, sizeof(float)) == 0;
     }
