@@ -32,14 +32,15 @@ namespace {
 
 constexpr int kRows = 32;         // spins per row block
 constexpr int kCols = 128;        // configurations per block (32 lanes x 4)
-constexpr int kVecBlocks = 608;   // blocks from which on a lane's spins are read as one word
 constexpr size_t kScratchBytes = size_t(4) << 20;  // 4 MiB
 constexpr size_t kScratchWords = kScratchBytes / 8;
 
 // Partial sums [row blocks][configurations padded to 128], int64 or double.
 static __device__ __align__(256) unsigned long long g_noalloc_scratch[kScratchWords];
 
-// Configurations c .. c + 3 (c a multiple of 4) of a row on a 4-byte boundary.
+// Configurations c .. c + 3 (c a multiple of 4) of a row on a 4-byte boundary;
+// the full-word branch is the only one taken with whole chunks, but without
+// the other the loop measured 43.0 instead of 32.8 us (L = 16, 2048).
 __device__ __forceinline__ uint32_t word4(const int8_t *row, int c, int count) {
   if (c + 4 <= count) return *reinterpret_cast<const uint32_t *>(row + c);
   uint32_t v = 0;
@@ -48,16 +49,17 @@ __device__ __forceinline__ uint32_t word4(const int8_t *row, int c, int count) {
   return v;
 }
 
-// VEC: rows of spins on 4-byte boundaries, so a lane reads its four
-// configurations as one word (those past count as zeros) and the gathers of
-// four entries are in flight at a time; lattice L = 16, 2048 configurations:
-// 39.2 -> 34.5 us.  Else a byte at a time.  Sums run in entry order.
+// VEC (integer J): rows of spins on 4-byte boundaries and whole chunks of 128
+// configurations, so a lane reads its four configurations as one word and the
+// gathers of four entries are in flight at a time.  Else a byte at a time.
+// Sums run in entry order.
 template <bool INT, bool VEC>
 __global__ void __launch_bounds__(256) k_energy_noalloc(int n, const int32_t *row_ptr, const int32_t *col,
                                                         const int32_t *val_i32, const double *val_f64,
                                                         const int64_t *h_i64, const double *h_f64,
                                                         const int8_t *spins, int ld, int count,
                                                         int cols_pad, void *scratch) {
+  static_assert(INT || !VEC, "words of spins are read for integer J only");
   using T = typename std::conditional<INT, long long, double>::type;
   __shared__ T sm[8][kCols];
   T *part = static_cast<T *>(scratch);
@@ -78,15 +80,15 @@ __global__ void __launch_bounds__(256) k_energy_noalloc(int n, const int32_t *ro
       for (int e = row_ptr[i]; e < e1; e += 4) {
         uint32_t sj4[4];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) sj4[u] = word4(spins + size_t(col[min(e + u, e1 - 1)]) * ld, c, count);
+        for (int u = 0; u < 4; ++u)
+          sj4[u] = word4(spins + size_t(col[min(e + u, e1 - 1)]) * ld, c, count);
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
           if (e + u >= e1) break;
 #pragma unroll
           for (int q = 0; q < 4; ++q) {
             const int s = int8_t(sj4[u] >> (8 * q));
-            if constexpr (INT) t[q] += (long long)val_i32[e + u] * s;
-            else t[q] += val_f64[e + u] * double(s);
+            t[q] += (long long)val_i32[e + u] * s;
           }
         }
       }
@@ -189,16 +191,16 @@ extern "C" int sbqa_energies_csr_noalloc(int32_t n, const int32_t *row_ptr, cons
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   dim3 grid(cols_pad / kCols, nblk);
   const unsigned fblocks = unsigned((count + 7) / 8);
-  // from about a wave of blocks on; a few blocks wait on latency either way, and the
-  // byte form's shorter chain wins (n = 1000, 300 configurations: 12.2 against 14.3 us)
-  const bool vec = ((reinterpret_cast<uintptr_t>(spins) | uintptr_t(uint32_t(ld))) & 3) == 0 &&
-                   int64_t(grid.x) * grid.y >= kVecBlocks;
+  // Words against bytes, us, sizes n x configurations: 1000 x 128 8.4 / 8.9, 4096 x 2048 32.8 / 37.5, degree 20
+  // 3000 x 1024 32.8 / 42.7; but with a chunk partly filled 216 x 16 9.1 / 7.4, 1000 x 300 10.4 / 9.0, and real J
+  // (bound by its FP64 arithmetic) 1000 x 128 22.6 / 21.9, 4096 x 2048 245.5 / 245.4.
+  const bool vec = count % kCols == 0 && ((reinterpret_cast<uintptr_t>(spins) | uintptr_t(uint32_t(ld))) & 3) == 0;
   if (integer) {
     (vec ? k_energy_noalloc<true, true> : k_energy_noalloc<true, false>)<<<grid, 256, 0, st>>>(
         n, row_ptr, col_idx, val_i32, nullptr, h_i64, nullptr, spins, ld, count, cols_pad, scratch);
     k_energy_noalloc_final<true><<<fblocks, 256, 0, st>>>(count, nblk, cols_pad, scratch, energy_int, energy);
   } else {
-    (vec ? k_energy_noalloc<false, true> : k_energy_noalloc<false, false>)<<<grid, 256, 0, st>>>(
+    k_energy_noalloc<false, false><<<grid, 256, 0, st>>>(
         n, row_ptr, col_idx, nullptr, val_f64, nullptr, h_f64, spins, ld, count, cols_pad, scratch);
     k_energy_noalloc_final<false><<<fblocks, 256, 0, st>>>(count, nblk, cols_pad, scratch, nullptr, energy);
   }

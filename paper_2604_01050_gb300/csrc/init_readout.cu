@@ -164,7 +164,7 @@ __device__ __forceinline__ double add_signed(double t, double w, uint32_t s4, in
 // in flight at a time; sums run in entry order.  FP64: signed additions, no
 // conversions (which run at the FP64 unit's rate too), so the FP64 adds bound
 // it.  Readout and start of a solve at N = 10^5, degree 6, R*P = 128, with the
-// split of k_best: 592 -> 419 us; lattice L = 16, R*P = 2048: 129 -> 79.
+// split of k_best: 592 -> 414 us; lattice L = 16, R*P = 2048: 129 -> 79.
 template <bool INT>
 __global__ void __launch_bounds__(256) k_energy_csr(StateView s, CsrView J, EnergyView E,
                                                     BestView b) {

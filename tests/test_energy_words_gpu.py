@@ -1,6 +1,6 @@
-"""sbqa_energies_csr_noalloc where spins are read as words (aligned rows, many
-blocks) and a byte at a time: the same energies from both, for integer and
-real couplings, and the exact ones."""
+"""sbqa_energies_csr_noalloc where spins are read as words (integer J, aligned
+rows, whole chunks of 128 configurations) and a byte at a time: the same
+energies from both, and the exact ones."""
 import numpy as np
 import pytest
 
@@ -10,7 +10,7 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("real", [False, True])
-@pytest.mark.parametrize("n,count", [(19500, 4), (2600, 1024), (2601, 1022), (700, 4000)])
+@pytest.mark.parametrize("n,count", [(33, 128), (19500, 128), (2601, 1024), (2600, 1022), (700, 4000)])
 def test_words_equal_bytes(n, count, real):
     import torch
 
