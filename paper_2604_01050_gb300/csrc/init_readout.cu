@@ -346,6 +346,8 @@ cudaError_t launch_energy_dense_fx(const StateView &s, const EnergyView &E, void
 // gather of N bytes).  From N = kBestSplit on the copy is a kernel of its own
 // over blocks of spins (N = 10^5, 8 runs: 190 us by 8 blocks).
 constexpr int kBestThreads = 256, kBestSplit = 16384;
+// have_best of a run: none yet (0), from an earlier readout, or from the last one
+constexpr int kBestKept = 1, kBestNew = 2;
 
 __global__ void __launch_bounds__(kBestThreads) k_best(StateView s, EnergyView E, BestView b, int step) {
   __shared__ int s_k;  // the winning replica, or -1 when the run does not improve
@@ -376,12 +378,12 @@ __global__ void __launch_bounds__(kBestThreads) k_best(StateView s, EnergyView E
       const bool have = b.have_best[r] != 0;
       const bool improve = !have || (E.is_integer ? ei < b.best_e_int[r] : ef < b.best_e[r]);
       s_k = improve ? k : -1;
+      b.have_best[r] = improve ? kBestNew : kBestKept;
       if (improve) {
         b.best_e_int[r] = E.is_integer ? ei : 0;
         b.best_e[r] = E.is_integer ? double(ei) : ef;
         b.best_k[r] = k;
         b.best_step[r] = step;
-        b.have_best[r] = 1;
       }
     }
   }
@@ -392,11 +394,11 @@ __global__ void __launch_bounds__(kBestThreads) k_best(StateView s, EnergyView E
   for (int i = threadIdx.x; i < s.N; i += kBestThreads) b.best_spins[size_t(r) * s.N + i] = s.Sg[size_t(i) * s.Cp + c];
 }
 
-// The spins of the runs that improved at this readout: their best is of `step`
-// (a run reads out once per step).
-__global__ void __launch_bounds__(kBestThreads) k_best_spins(StateView s, BestView b, int step) {
+// The spins of the runs that improved at this readout.  (Not told by their
+// step: after sbqa_set_state a run may read out at the same step again.)
+__global__ void __launch_bounds__(kBestThreads) k_best_spins(StateView s, BestView b) {
   const int r = blockIdx.x;
-  if (b.best_step[r] != step) return;
+  if (b.have_best[r] != kBestNew) return;
   const int c = r * s.P + b.best_k[r], i = blockIdx.y * kBestThreads + threadIdx.x;
   if (i < s.N) b.best_spins[size_t(r) * s.N + i] = s.Sg[size_t(i) * s.Cp + c];
 }
@@ -405,7 +407,7 @@ cudaError_t launch_best(const StateView &s, const EnergyView &E, const BestView 
                         cudaStream_t st) {
   k_best<<<s.R, kBestThreads, 0, st>>>(s, E, b, step);
   if (s.N >= kBestSplit)
-    k_best_spins<<<dim3(s.R, (s.N + kBestThreads - 1) / kBestThreads), kBestThreads, 0, st>>>(s, b, step);
+    k_best_spins<<<dim3(s.R, (s.N + kBestThreads - 1) / kBestThreads), kBestThreads, 0, st>>>(s, b);
   return cudaGetLastError();
 }
 

@@ -101,7 +101,7 @@ struct BestView {
   int32_t *best_k;       // [R]
   int32_t *best_step;    // [R]
   int8_t *best_spins;    // [R][N]
-  int32_t *have_best;    // [R]
+  int32_t *have_best;    // [R] 0: none yet, kBestKept or kBestNew (init_readout.cu)
 };
 
 // Records msg as the calling thread's detail message (sbqa_last_error) and
