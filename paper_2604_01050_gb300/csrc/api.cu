@@ -642,23 +642,30 @@ int prepare_tc_values(sbqa_problem *p) {
 }
 
 // The fixed-point readout operands of a real J, from its FP64 copy on the
-// device.  Without the memory for them (or with row sums past the FP64 range)
-// the FP64 readout on the CUDA cores serves.
+// device.  Without the memory for them, or where the fixed point would be the
+// less accurate form, the FP64 readout on the CUDA cores serves.
 int prepare_fx(sbqa_problem *p) {
   if (p->fx_tried || p->is_integer || !fx_eligible(p->n)) return SBQA_OK;
+  DevBuf<double> scratch;
+  if (scratch.alloc(size_t(2) * p->n) != cudaSuccess) {
+    cudaGetLastError();
+    return SBQA_OK;
+  }
+  int k = 0;
+  bool serves = false;
+  const cudaError_t e = fx_choose(p->d_e_f64.p, p->h.empty() ? nullptr : p->h.data(), p->n, scratch.p, &k, &serves,
+                                  nullptr);
+  scratch.release(true);
+  SBQA_CUDA(e);
   p->fx_tried = true;
-  DevBuf<unsigned long long> scratch;
-  if (p->d_fx_digits.alloc(fx_digit_bytes(p->n)) != cudaSuccess || p->d_fx_h.alloc(p->n) != cudaSuccess ||
-      scratch.alloc(1) != cudaSuccess) {
+  if (!serves) return SBQA_OK;
+  if (p->d_fx_digits.alloc(fx_digit_bytes(p->n)) != cudaSuccess || p->d_fx_h.alloc(p->n) != cudaSuccess) {
     cudaGetLastError();
     p->d_fx_digits.release();
     p->d_fx_h.release();
     return SBQA_OK;
   }
-  const cudaError_t e = fx_plan_make(&p->fx_plan, p->d_e_f64.p, p->d_h_f64.p, p->n, p->d_fx_digits.p, p->d_fx_h.p,
-                                     scratch.p, nullptr);
-  scratch.release(true);
-  SBQA_CUDA(e);
+  SBQA_CUDA(fx_plan_make(&p->fx_plan, p->d_e_f64.p, p->d_h_f64.p, p->n, k, p->d_fx_digits.p, p->d_fx_h.p, nullptr));
   return SBQA_OK;
 }
 

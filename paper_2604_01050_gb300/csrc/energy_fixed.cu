@@ -11,13 +11,21 @@
 // sums of a tile (below 2^24 in FP32), which the epilogue joins as
 // acc = 256 acc + digit in 64-bit integers.  Rows and then row blocks add as
 // integers too (the 64-bit values in two 32-bit halves), so the only roundings
-// are those of X and H and one of the result: an energy is closer to the
-// instance's than the FP64 sum in any order, whatever the order.
+// are those of X and H and one of the result.
+//
+// One unit 2^-k serves the whole instance, so what is small beside the largest
+// row sum is held in few bits, where an FP64 sum would keep it: a spin pinned
+// by a large field, say.  The plan is therefore made only where the error is
+// no larger than that of the FP64 sums (fx_scale); elsewhere they serve.  For
+// Gaussian J of N = 64 .. 2048 the error is 0.36 to 0.46 of theirs (root mean
+// square), with fields of up to the size of the row sums 0.55 to 0.61.
 // At N = 2000, R*P = 1024 the eight GEMMs (66 GFLOP, operands 64 MB, in L2)
 // and the kernels around them take 0.14 ms instead of 10.7; at N = 1000, R*P =
 // 256 the readout takes 0.04 ms instead of 1.34.
+#include <algorithm>
 #include <cmath>
 #include <cstdint>
+#include <vector>
 
 #include "dense_tc_common.cuh"
 
@@ -32,20 +40,39 @@ struct FxPlan {
   int k, Kp;
 };
 
-// Largest row sum of |J_ij| + 2 |h_i| (bits of a non-negative double, which
-// order as integers do).
-__global__ void __launch_bounds__(256) k_fx_rowsum(const double *J, const double *h, int N, unsigned long long *most) {
+// Per row, for the choice of the scale: A_i = sum_j |J_ij|, and q_i = sum_j
+// (N - j) J_ij^2 in units of 2^(2 ilogb(A_i)), to a few per mille: the leading 21 bits
+// of each entry, by its exponent field, as a float (no FP64 arithmetic;
+// subnormal entries count as 0).
+__global__ void __launch_bounds__(256) k_fx_rows(const double *J, int N, double *A, double *q) {
   __shared__ double sm[8];
+  __shared__ float sq[8];
+  __shared__ int s_e;
   const int i = blockIdx.x;
+  const double *row = J + size_t(i) * N;
   double acc = 0.0;
-  for (int j = threadIdx.x; j < N; j += 256) acc += fabs(J[size_t(i) * N + j]);
+  for (int j = threadIdx.x; j < N; j += 256) acc += fabs(row[j]);
   for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
   if ((threadIdx.x & 31) == 0) sm[threadIdx.x >> 5] = acc;
   __syncthreads();
   if (threadIdx.x == 0) {
     for (int w = 1; w < 8; ++w) acc += sm[w];
-    acc += 2.0 * fabs(h[i]);
-    atomicMax(most, static_cast<unsigned long long>(__double_as_longlong(acc)));
+    A[i] = acc;
+    s_e = (__double2hiint(acc) >> 20) & 0x7ff;  // not 0x7ff: the host refuses infinite sums whatever q is
+  }
+  __syncthreads();
+  float w2 = 0.f;
+  for (int j = threadIdx.x; j < N; j += 256) {
+    const int hi = __double2hiint(row[j]), field = (hi >> 20) & 0x7ff, e = field - s_e + 127;
+    const float v = field > 0 && e > 0 ? __uint_as_float(uint32_t(e) << 23 | uint32_t(hi & 0xfffff) << 3) : 0.f;
+    w2 = fmaf(v * v, float(N - j), w2);
+  }
+  for (int o = 16; o > 0; o >>= 1) w2 += __shfl_down_sync(0xffffffffu, w2, o);
+  if ((threadIdx.x & 31) == 0) sq[threadIdx.x >> 5] = w2;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < 8; ++w) w2 += sq[w];
+    q[i] = w2;
   }
 }
 
@@ -254,27 +281,70 @@ size_t fx_spin_bytes(int N, int Cp) { return size_t(Cp) * tc_padded(N) * 2; }
 // spins would not fit the buffers they are given.
 bool fx_eligible(int N) { return N >= 64 && tc_padded(N) <= kFxMaxKp; }
 
-cudaError_t fx_plan_make(void **plan, const double *J, const double *h, int N, void *digits, int64_t *H,
-                         unsigned long long *scratch, cudaStream_t st) {
+// Whether the fixed point serves, and its scale k: row sums |J_i| + 2 |h_i|
+// below 2^62 after scaling.  The energies' root mean square errors, for spins
+// of random signs: here N^2 / 2 pairs rounded to units u = 2^-k, 0.20 N u; in
+// FP64, a rounding of 0.43 2^-53 of each partial sum along a row (variance
+// sum_{l <= j} J_il^2 after entry j; halved in the energy) and of each row's
+// field, 0.21 2^-53 sqrt(sum_i q_i + 4 sum_i h_i^2).  N counts the rows that are
+// not empty, and both sums are taken as N times the median one's, so that a few large rows or fields, which may cancel
+// in FP64 and leave the others' sums intact, do not stand for the rest.  The
+// line lies where the two are equal, which favours FP64: aligned spins make
+// its partial sums larger.  (One row 10^4 times the others at N = 300 and
+// fields of N times the couplings at N = 2048, on either side of the line:
+// 0.24 and 0.55 of the FP64 error.)
+static bool fx_scale(const std::vector<double> &A, const std::vector<double> &q, const double *h, int N, int *k) {
+  double most = 0.0, largest = 0.0;
+  for (int i = 0; i < N; ++i) {
+    largest = std::max(largest, A[i]);
+    most = std::max(most, A[i] + (h ? 2.0 * std::fabs(h[i]) : 0.0));
+  }
+  if (!std::isfinite(most)) return false;
+  *k = most > 0.0 ? 61 - std::ilogb(most) : 0;
+  if (most == 0.0) return true;
+  // in units of 2^e, so that no square leaves the FP64 range
+  const int e = std::ilogb(largest > 0.0 ? largest : most);
+  auto median = [](std::vector<double> &v) {
+    auto mid = v.begin() + v.size() / 2;
+    std::nth_element(v.begin(), mid, v.end());
+    return *mid;
+  };
+  std::vector<double> rq, rh;
+  for (int i = 0; i < N; ++i) {
+    if (A[i] == 0.0 && (!h || h[i] == 0.0)) continue;
+    rq.push_back(A[i] > 0.0 ? std::ldexp(q[i], 2 * (std::ilogb(A[i]) - e)) : 0.0);
+    rh.push_back(h ? std::fabs(std::ldexp(h[i], -e)) : 0.0);
+  }
+  const double mq = median(rq), mh = median(rh);
+  return std::sqrt(double(rq.size())) * std::ldexp(1.0, -*k - e) <= std::ldexp(std::sqrt(mq + 4.0 * mh * mh), -53);
+}
+
+cudaError_t fx_choose(const double *J, const double *h_host, int N, double *scratch, int *k, bool *serves,
+                      cudaStream_t st) {
+  *serves = false;
+  k_fx_rows<<<N, 256, 0, st>>>(J, N, scratch, scratch + N);
+  std::vector<double> A(N), q(N);
+  cudaError_t e = cudaGetLastError();
+  if (e == cudaSuccess) e = cudaMemcpyAsync(A.data(), scratch, N * sizeof(double), cudaMemcpyDeviceToHost, st);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(q.data(), scratch + N, N * sizeof(double), cudaMemcpyDeviceToHost, st);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+  if (e == cudaSuccess) *serves = fx_scale(A, q, h_host, N, k);
+  return e;
+}
+
+cudaError_t fx_plan_make(void **plan, const double *J, const double *h, int N, int k, void *digits, int64_t *H,
+                         cudaStream_t st) {
   const int Kp = tc_padded(N);
   *plan = nullptr;
   cudaError_t e = cudaFuncSetAttribute((const void *)k_energy_dense_fx, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        kFxSmem);
-  if (e == cudaSuccess) e = cudaMemsetAsync(scratch, 0, sizeof(*scratch), st);
   if (e != cudaSuccess) return e;
-  k_fx_rowsum<<<N, 256, 0, st>>>(J, h, N, scratch);
-  double most = 0.0;
-  if ((e = cudaGetLastError()) != cudaSuccess ||
-      (e = cudaMemcpyAsync(&most, scratch, sizeof(most), cudaMemcpyDeviceToHost, st)) != cudaSuccess ||
-      (e = cudaStreamSynchronize(st)) != cudaSuccess)
-    return e;
-  if (!std::isfinite(most)) return cudaSuccess;  // row sums past the FP64 range: no plan
   auto *p = new FxPlan();
-  p->k = most > 0.0 ? 61 - std::ilogb(most) : 0;  // row sums below 2^62 after scaling
+  p->k = k;
   p->H = H;
   p->Kp = Kp;
   const size_t total = size_t(Kp) * Kp;
-  k_fx_digits<<<unsigned((total + 255) / 256), 256, 0, st>>>(J, h, N, Kp, p->k, static_cast<uint16_t *>(digits), H);
+  k_fx_digits<<<unsigned((total + 255) / 256), 256, 0, st>>>(J, h, N, Kp, k, static_cast<uint16_t *>(digits), H);
   e = cudaGetLastError();
   if (e == cudaSuccess && !tc_make_map(&p->A, digits, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, uint64_t(kFxDigits) * Kp,
                                        uint64_t(Kp), 64, 128, CU_TENSOR_MAP_SWIZZLE_128B))

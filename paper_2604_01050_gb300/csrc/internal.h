@@ -367,13 +367,16 @@ cudaError_t launch_energy_dense_tc(const void *plan, const StateView &s, int Kp,
 // Readout energies of a real dense instance on the tensor cores: J and h in
 // 64-bit fixed point, one bfloat16 operand per byte (energy_fixed.cu).  The
 // plan is made once per problem from the FP64 J [N][N] and h [N] into digits
-// (fx_digit_bytes) and H [N]; *plan stays null when the row sums leave the
-// FP64 range.  The spins take fx_spin_bytes at `spins` (16-byte aligned).
+// (fx_digit_bytes) and H [N], with the scale k of fx_choose where that says
+// that the fixed point serves (scratch [2 N]; h on the host, or null for 0).
+// The spins take fx_spin_bytes at `spins` (16-byte aligned).
 bool fx_eligible(int N);
 size_t fx_digit_bytes(int N);
 size_t fx_spin_bytes(int N, int Cp);
-cudaError_t fx_plan_make(void **plan, const double *J, const double *h, int N, void *digits, int64_t *H,
-                         unsigned long long *scratch, cudaStream_t st);
+cudaError_t fx_choose(const double *J, const double *h_host, int N, double *scratch, int *k, bool *serves,
+                      cudaStream_t st);
+cudaError_t fx_plan_make(void **plan, const double *J, const double *h, int N, int k, void *digits, int64_t *H,
+                         cudaStream_t st);
 void fx_plan_free(void *plan);
 cudaError_t launch_energy_partials_fx(const void *fx_plan, const StateView &s, void *spins, int *err,
                                       const BestView &best, cudaStream_t st);
