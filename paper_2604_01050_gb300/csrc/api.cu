@@ -1985,7 +1985,7 @@ int sbqa_run(sbqa_problem *p, int32_t steps, int32_t P, int32_t R, uint64_t seed
   }
   sbqa_problem::Key key;
   key.S = steps; key.P = P; key.R = R; key.eval = p->prm.eval_every; key.kind = p->kind;
-  key.dense = p->dense ? 1 : 0; key.x = p->d_x.p; key.kj = p->d_kj.p; key.results = p->d_results.p;
+  key.dense = p->dense ? 1 : 0; key.moves = p->buffer_moves();
   key.kc = p->tables.kc; key.kx = p->tables.kx; key.tc = p->use_tc ? 1 + p->tc_op : 0; key.variant = p->csr_variant;
   key.fvar = p->prm.variant;
   if (!(p->graph && p->graph_key == key)) {

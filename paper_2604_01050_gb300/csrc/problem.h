@@ -74,6 +74,7 @@ struct DevBuf {
   T *p = nullptr;
   size_t n = 0;      // elements the block holds (at least the count asked for)
   size_t bytes = 0;  // its size class
+  uint64_t moves = 0;  // blocks taken so far: the address is the same while this is
   cudaError_t alloc(size_t count) {
     if (count <= n && p) return cudaSuccess;
     release();
@@ -85,6 +86,7 @@ struct DevBuf {
     p = static_cast<T *>(q);
     n = got / sizeof(T);
     bytes = got;
+    ++moves;
     return cudaSuccess;
   }
   // idle: the caller has synchronized the device, so no work still uses the
@@ -258,13 +260,23 @@ struct sbqa_problem {
   struct Key {
     int S = -1, P = -1, R = -1, eval = -1, kind = -1, dense = -1, tc = -1, variant = -1, fvar = -1;
     float kc = 0.f, kx = 0.f;  // step constants are kernel arguments in the graph
-    const void *x = nullptr, *kj = nullptr, *results = nullptr;
+    uint64_t moves = 0;        // ... and so are the addresses of the handle's buffers
     bool operator==(const Key &o) const {
-      return S == o.S && P == o.P && R == o.R && results == o.results && eval == o.eval && kind == o.kind &&
-             dense == o.dense && tc == o.tc && variant == o.variant && fvar == o.fvar && x == o.x && kj == o.kj &&
+      return S == o.S && P == o.P && R == o.R && moves == o.moves && eval == o.eval && kind == o.kind &&
+             dense == o.dense && tc == o.tc && variant == o.variant && fvar == o.fvar &&
              std::memcmp(&kc, &o.kc, sizeof(float)) == 0 && std::memcmp(&kx, &o.kx, sizeof(float)) == 0;
     }
   } graph_key;
+
+  // Grows whenever a buffer that a launch may name has moved.  A graph names them all, and they move one
+  // by one: each keeps its block while the new size fits the block's size class.
+  uint64_t buffer_moves() const {
+    auto sum = [](const auto &...b) { return (uint64_t(0) + ... + b.moves); };
+    return sum(d_jcopy_i8, d_row_ptr, d_col, d_col_pm1, d_npos, d_val_f32, d_val_bf16, d_dense_f32, d_J8, d_FT,
+               d_results, d_h, d_e_i32, d_e_f64, d_h_i64, d_h_f64, d_fx_digits, d_fx_h, d_fx_spins, d_bar, d_tc_flags,
+               d_J4, d_FT4, d_x, d_y, d_F0, d_F1, d_ell_col, d_ell_meta, d_ell_val, d_Fx0, d_Fx1, d_Sg, d_ka, d_dl,
+               d_kj, d_part_i, d_part_f, d_have);
+  }
 
   ~sbqa_problem();  // waits for the device, releases every buffer (api.cu)
 
