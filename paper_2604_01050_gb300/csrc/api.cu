@@ -165,6 +165,21 @@ void sbqa::hostcache_put(void *p, size_t bytes) {
   c.held += cls;
 }
 
+// Test hook: SBQA_TEST_FAIL_ALLOC=bytes:count makes the next `count` requests of at least `bytes` bytes
+// fail as on a full device, counted from when the variable is set (not for production use).  The caller
+// holds the lock.
+static bool fail_alloc_hook(size_t bytes) {
+  static std::string seen;
+  static size_t least = 0;
+  static int left = 0;
+  const char *v = std::getenv("SBQA_TEST_FAIL_ALLOC");
+  if (seen != (v ? v : "")) {
+    seen = v ? v : "";
+    if (std::sscanf(seen.c_str(), "%zu:%d", &least, &left) != 2) left = 0;
+  }
+  return left > 0 && bytes >= least && left-- > 0;
+}
+
 cudaError_t sbqa::devcache_get(void **p, size_t bytes, size_t *got) {
   const size_t cls = size_class(bytes);
   int dev = 0;
@@ -173,6 +188,10 @@ cudaError_t sbqa::devcache_get(void **p, size_t bytes, size_t *got) {
   DevCache &c = devcache();
   {
     std::lock_guard<std::mutex> lk(c.mu);
+    if (fail_alloc_hook(bytes)) {
+      *p = nullptr;
+      return cudaErrorMemoryAllocation;
+    }
     auto &m = c.blocks[dev];
     auto it = m.find(cls);
     if (it != m.end()) {
@@ -193,6 +212,7 @@ cudaError_t sbqa::devcache_get(void **p, size_t bytes, size_t *got) {
     e = cudaMalloc(p, cls);
   }
   if (e != cudaSuccess) {
+    cudaGetLastError();  // reported here, and not again by the next launch
     *p = nullptr;
     return e;
   }
@@ -782,7 +802,14 @@ struct ResultLayout {
 cudaError_t carve_results(sbqa_problem *p, int R, int Cp) {
   const ResultLayout l(size_t(p->n), size_t(R), size_t(Cp));
   const cudaError_t e = p->d_results.alloc(l.end);
-  if (e != cudaSuccess) return e;
+  if (e != cudaSuccess) {  // the block before is gone too: no part of it is left to be read
+    p->d_err.p = nullptr;
+    p->d_best_e.p = p->d_ef.p = nullptr;
+    p->d_best_ei.p = p->d_ei.p = nullptr;
+    p->d_best_k.p = p->d_best_step.p = nullptr;
+    p->d_best_spins.p = nullptr;
+    return e;
+  }
   uint8_t *b = p->d_results.p;
   p->d_err.p = reinterpret_cast<int *>(b);
   p->d_best_e.p = reinterpret_cast<double *>(b + l.best_e);
