@@ -661,9 +661,45 @@ int prepare_tc_values(sbqa_problem *p) {
   return SBQA_OK;
 }
 
+// Planes of this size and more (N = 4096) are taken only while they are an
+// eighth of the free memory at most, so that other handles fit which would fit
+// without them.
+constexpr size_t kFxLargePlanes = size_t(256) << 20;
+
+bool fx_planes_fit(size_t bytes) {
+  if (bytes < kFxLargePlanes) return true;
+  size_t free_bytes = 0, total = 0;
+  if (cudaMemGetInfo(&free_bytes, &total) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return bytes <= free_bytes / 8;
+}
+
+// Gives up the fixed-point readout of the handle; the FP64 one serves from then on.
+void release_fx(sbqa_problem *p) {
+  p->d_fx_digits.release();  // waits for the device: no readout still uses the plan
+  p->d_fx_h.release(true);
+  p->d_fx_spins.release(true);
+  if (p->fx_plan) fx_plan_free(p->fx_plan);
+  p->fx_plan = nullptr;
+}
+
+// work(), and where that runs out of device memory once more without the
+// planes of the fixed-point readout: they must not keep out a run that fits
+// without them.
+template <class Work>
+int with_fx_memory(sbqa_problem *p, Work work) {
+  const int rc = work();
+  if (rc != SBQA_ERR_OOM || !p->fx_plan) return rc;
+  release_fx(p);
+  return work();
+}
+
 // The fixed-point readout operands of a real J, from its FP64 copy on the
-// device.  Without the memory for them, or where the fixed point would be the
-// less accurate form, the FP64 readout on the CUDA cores serves.
+// device: 16 bytes per coupling, for the life of the handle.  Without the
+// memory for them, or where the fixed point would be the less accurate form,
+// the FP64 readout on the CUDA cores serves.
 int prepare_fx(sbqa_problem *p) {
   if (p->fx_tried || p->is_integer || !fx_eligible(p->n)) return SBQA_OK;
   DevBuf<double> scratch;
@@ -678,7 +714,7 @@ int prepare_fx(sbqa_problem *p) {
   scratch.release(true);
   SBQA_CUDA(e);
   p->fx_tried = true;
-  if (!serves) return SBQA_OK;
+  if (!serves || !fx_planes_fit(fx_digit_bytes(p->n))) return SBQA_OK;
   if (p->d_fx_digits.alloc(fx_digit_bytes(p->n)) != cudaSuccess || p->d_fx_h.alloc(p->n) != cudaSuccess) {
     cudaGetLastError();
     p->d_fx_digits.release();
@@ -1457,7 +1493,9 @@ int sbqa::problem_check_run(sbqa_problem *p, int32_t steps, int32_t P, int32_t R
 
 int sbqa::problem_prepare_values(sbqa_problem *p) {
   DeviceGuard g(p->device);
-  return p->dense ? prepare_dense_values(p, p->prm.precision) : prepare_sparse_values(p, p->prm.precision);
+  return with_fx_memory(p, [&] {
+    return p->dense ? prepare_dense_values(p, p->prm.precision) : prepare_sparse_values(p, p->prm.precision);
+  });
 }
 
 // FP64 schedule of Sec. II A rounded to the FP32 step coefficients.
@@ -1923,15 +1961,8 @@ int sbqa_set_schedule(sbqa_problem *p, const sbqa_params *q) {
   return SBQA_OK;
 }
 
-int sbqa_run_begin(sbqa_problem *p, int32_t steps, int32_t P, int32_t R, uint64_t seed, void *stream) {
-  int rc = check_run_args(p, steps, P, R);
-  if (rc != SBQA_OK) return rc;
-  DeviceGuard g(p->device);
-  p->small_path = false;
-  p->wide_x = false;
-  p->stream = static_cast<cudaStream_t>(stream);
-  p->begun = p->finished = false;
-  rc = p->dense ? prepare_dense_values(p, p->prm.precision) : prepare_sparse_values(p, p->prm.precision);
+static int begin_run(sbqa_problem *p, int32_t steps, int32_t P, int32_t R, uint64_t seed) {
+  int rc = p->dense ? prepare_dense_values(p, p->prm.precision) : prepare_sparse_values(p, p->prm.precision);
   if (rc != SBQA_OK) return rc;
   if ((rc = alloc_run(p, steps, P, R)) != SBQA_OK) return rc;
   if ((rc = build_tables(p)) != SBQA_OK) return rc;
@@ -1947,6 +1978,17 @@ int sbqa_run_begin(sbqa_problem *p, int32_t steps, int32_t P, int32_t R, uint64_
   p->step_done = 0;
   p->begun = true;
   return SBQA_OK;
+}
+
+int sbqa_run_begin(sbqa_problem *p, int32_t steps, int32_t P, int32_t R, uint64_t seed, void *stream) {
+  const int rc = check_run_args(p, steps, P, R);
+  if (rc != SBQA_OK) return rc;
+  DeviceGuard g(p->device);
+  p->small_path = false;
+  p->wide_x = false;
+  p->stream = static_cast<cudaStream_t>(stream);
+  p->begun = p->finished = false;
+  return with_fx_memory(p, [&] { return begin_run(p, steps, P, R, seed); });
 }
 
 int sbqa_run_advance(sbqa_problem *p, int32_t n_steps) {

@@ -180,7 +180,8 @@ struct sbqa_problem {
   sbqa::DevBuf<double> d_e_f64;
   sbqa::DevBuf<int64_t> d_h_i64;
   sbqa::DevBuf<double> d_h_f64;
-  // fixed-point readout of a real dense J (energy_fixed.cu); made once
+  // fixed-point readout of a real dense J (energy_fixed.cu); made once, given up for a run that does not
+  // fit beside it
   sbqa::DevBuf<uint8_t> d_fx_digits;
   sbqa::DevBuf<int64_t> d_fx_h;
   void *fx_plan = nullptr;

@@ -25,9 +25,13 @@ def _gauss(sb, n, **kw):
 
 
 def test_a_handle_whose_results_did_not_fit(sb, monkeypatch):
-    """Same columns, more runs: only the block of the results (300 KB) has to grow, and does not get the
-    memory.  The handle has no results then, synchronises, and solves once there is memory again."""
-    pb = _gauss(sb, 300)
+    """Same columns, more runs: only the block of the results (200 KB) has to grow, and does not get the
+    memory.  The handle has no results then, synchronises, and solves once there is memory again.
+    (Integer couplings: no planes to give up for it.)"""
+    up = np.triu(np.random.default_rng(1).integers(-3, 4, (200, 200)).astype(float), 1)
+    pb, fresh = (sb.create_problem_dense(up + up.T) for _ in range(2))
+    sb.set_schedule(pb)
+    sb.set_schedule(fresh)
     sb.run(pb, 2, 128, 8, seed=1)
     monkeypatch.setenv("SBQA_TEST_FAIL_ALLOC", "100000:1")
     with pytest.raises(sb.SBQAError) as e:
@@ -39,8 +43,36 @@ def test_a_handle_whose_results_did_not_fit(sb, monkeypatch):
         sb.get_best(pb)
     assert e.value.status == sb.ERR_STATE
     sb.run(pb, 2, 1, 1000, seed=2)
-    fresh = _gauss(sb, 300)
     sb.run(fresh, 2, 1, 1000, seed=2)
     a, b = sb.get_best(pb), sb.get_best(fresh)
     for k in a:
         assert np.array_equal(a[k], b[k]), k
+
+
+@pytest.mark.parametrize("failures", ["6500000:1", "2000000:1"])
+def test_the_readout_planes_keep_no_run_out(sb, monkeypatch, failures):
+    """The planes of the fixed-point readout (6.6 MB) do not fit, or a larger run (2.6 MB of positions)
+    does not fit beside them: the FP64 readout serves, to the same spins."""
+    fresh = _gauss(sb, 640, gamma0=32.0)
+    sb.run(fresh, 30, 8, 128, seed=2)
+    a, ea = sb.get_best(fresh), sb.get_energies(fresh)[0]
+    pb = _gauss(sb, 640, gamma0=32.0)
+    if failures.startswith("2"):
+        sb.run(pb, 30, 8, 4, seed=1)
+    monkeypatch.setenv("SBQA_TEST_FAIL_ALLOC", failures)
+    for again in range(2):  # the second time the kept graph
+        sb.run(pb, 30, 8, 128, seed=2)
+        b, eb = sb.get_best(pb), sb.get_energies(pb)[0]
+        assert np.array_equal(a["spins"], b["spins"]) and np.array_equal(a["replica"], b["replica"])
+        assert np.allclose(ea, eb, rtol=1e-12, atol=1e-9) and not np.array_equal(ea, eb)
+
+
+def test_a_run_that_does_not_fit_without_the_planes_either(sb, monkeypatch):
+    pb = _gauss(sb, 640, gamma0=32.0)
+    sb.run(pb, 30, 8, 4, seed=1)
+    monkeypatch.setenv("SBQA_TEST_FAIL_ALLOC", "2000001:2")
+    with pytest.raises(sb.SBQAError) as e:
+        sb.run(pb, 30, 8, 128, seed=2)
+    assert e.value.status == sb.ERR_OOM
+    sb.run(pb, 30, 8, 128, seed=2)
+    assert np.isfinite(sb.get_best(pb)["energy"]).all()
