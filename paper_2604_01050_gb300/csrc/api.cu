@@ -1468,19 +1468,27 @@ int check_run_args(sbqa_problem *p, int32_t steps, int32_t P, int32_t R) {
 // The caller's state arrays [R * P][N] pass through the device in slices of
 // whole replicas (at most 32 MiB, one replica at least), where a kernel
 // changes the layout; the slice comes from the block cache and goes back to
-// it.  Its last words take two flags.
+// it.  Without memory for it the signs' buffer serves, which holds N bytes per
+// column (30 replicas and more) and nothing between two readouts.  Behind the
+// slice one word takes a flag.
 struct StateSlices {
   const sbqa_problem *p;
   int replicas, per_slice;
-  DevBuf<float> rows;
+  DevBuf<float> block;
+  float *rows;
   explicit StateSlices(const sbqa_problem *q) : p(q), replicas(q->R * q->P) {
-    const int64_t fit = (int64_t(8) << 20) / std::max(1, q->n);
-    per_slice = int(std::max<int64_t>(1, std::min<int64_t>(fit, replicas)));
+    const int64_t n = q->n, fit = std::max<int64_t>(1, (int64_t(8) << 20) / n);
+    per_slice = int(std::min<int64_t>(fit, replicas));
+    if (block.alloc(size_t(per_slice) * n + 1) == cudaSuccess) {
+      rows = block.p;
+    } else {
+      rows = reinterpret_cast<float *>(q->d_Sg.p);
+      per_slice = int(std::min<int64_t>(per_slice, (n * q->Cp / 4 - 1) / n));
+    }
   }
-  cudaError_t alloc() { return rows.alloc(size_t(per_slice) * p->n + 2); }
   ~StateSlices() {
-    if (rows.p) cudaStreamSynchronize(p->stream);  // also after an error: nothing uses the slice any more
-    rows.release(true);
+    cudaStreamSynchronize(p->stream);  // also after an error: nothing uses the slice any more
+    block.release(true);
   }
 };
 
@@ -2145,14 +2153,13 @@ int sbqa_get_state(sbqa_problem *p, float *x, float *y, int32_t *step_done) {
   if (rc != SBQA_OK) return rc;
   DeviceGuard g(p->device);
   StateSlices sl(p);
-  SBQA_CUDA(sl.alloc());
   float *outs[2] = {x, y}, *src[2] = {p->d_x.p, p->d_y.p};
   for (int w = 0; w < 2; ++w) {
     if (!outs[w]) continue;
     for (int q0 = 0; q0 < sl.replicas; q0 += sl.per_slice) {
       const int count = std::min(sl.per_slice, sl.replicas - q0);
-      SBQA_CUDA(launch_state_rows(p->state(), src[w], sl.rows.p, q0, count, true, nullptr, p->stream));
-      SBQA_CUDA(cudaMemcpyAsync(outs[w] + size_t(q0) * p->n, sl.rows.p, size_t(count) * p->n * sizeof(float),
+      SBQA_CUDA(launch_state_rows(p->state(), src[w], sl.rows, q0, count, true, nullptr, p->stream));
+      SBQA_CUDA(cudaMemcpyAsync(outs[w] + size_t(q0) * p->n, sl.rows, size_t(count) * p->n * sizeof(float),
                                 cudaMemcpyDeviceToHost, p->stream));
       SBQA_CUDA(cudaStreamSynchronize(p->stream));
     }
@@ -2169,26 +2176,24 @@ int sbqa_set_state(sbqa_problem *p, const float *x, const float *y, int32_t step
   if (rc != SBQA_OK) return rc;
   DeviceGuard g(p->device);
   StateSlices sl(p);
-  SBQA_CUDA(sl.alloc());
   const size_t NC = size_t(p->n) * p->Cp;
   const float *in[2] = {x, y};
   float *dst[2] = {p->d_x.p, p->d_y.p};
-  int *wide = reinterpret_cast<int *>(sl.rows.p + size_t(sl.per_slice) * p->n);  // of x, then of y
-  int is_wide[2] = {0, 0};
-  SBQA_CUDA(cudaMemsetAsync(wide, 0, sizeof(is_wide), p->stream));
+  int *wide = reinterpret_cast<int *>(sl.rows + size_t(sl.per_slice) * p->n), is_wide = 0;
+  SBQA_CUDA(cudaMemsetAsync(wide, 0, sizeof(int), p->stream));
   for (int w = 0; w < 2; ++w) {
     SBQA_CUDA(cudaMemsetAsync(dst[w], 0, NC * sizeof(float), p->stream));  // padding columns of a run stay at zero
     for (int q0 = 0; q0 < sl.replicas; q0 += sl.per_slice) {
       const int count = std::min(sl.per_slice, sl.replicas - q0);
-      SBQA_CUDA(cudaMemcpyAsync(sl.rows.p, in[w] + size_t(q0) * p->n, size_t(count) * p->n * sizeof(float),
+      SBQA_CUDA(cudaMemcpyAsync(sl.rows, in[w] + size_t(q0) * p->n, size_t(count) * p->n * sizeof(float),
                                 cudaMemcpyHostToDevice, p->stream));
-      SBQA_CUDA(launch_state_rows(p->state(), dst[w], sl.rows.p, q0, count, false, wide + w, p->stream));
+      SBQA_CUDA(launch_state_rows(p->state(), dst[w], sl.rows, q0, count, false, w == 0 ? wide : nullptr, p->stream));
       SBQA_CUDA(cudaStreamSynchronize(p->stream));
     }
   }
-  SBQA_CUDA(cudaMemcpyAsync(is_wide, wide, sizeof(is_wide), cudaMemcpyDeviceToHost, p->stream));
+  SBQA_CUDA(cudaMemcpyAsync(&is_wide, wide, sizeof(int), cudaMemcpyDeviceToHost, p->stream));
   SBQA_CUDA(cudaStreamSynchronize(p->stream));
-  p->wide_x = is_wide[0] != 0;
+  p->wide_x = is_wide != 0;
   const double tau = p->S > 0 ? double(step_done) / double(p->S) : 0.0;
   SBQA_CUDA(launch_refresh_f(p->state(), step_done & 1, float(p->prm.delta_slope * tau), p->stream));
   if (p->use_tc)

@@ -77,7 +77,7 @@ cudaError_t launch_refresh_f(const StateView &s, int which, float delta, cudaStr
 // caller's [R * Pr][N] (replica q = r * Pr + k), through 32 x 32 tiles so that
 // both sides are coalesced.  On the host the same gather, one element per
 // cache line, took 2.5 ns per value.  OUT: to the caller; else from it, *wide
-// set when some |v| >= 2 or NaN.
+// (unless null) set when some |v| >= 2 or NaN.
 template <bool OUT>
 __global__ void __launch_bounds__(256) k_state_layout(float *v, float *rows, int N, int Cp, int P, int Pr, int q0,
                                                       int count, int *wide) {
@@ -98,7 +98,7 @@ __global__ void __launch_bounds__(256) k_state_layout(float *v, float *rows, int
         t[a][r] = x;
         big = big || !(fabsf(x) < 2.f);
       }
-    if (big) *wide = 1;
+    if (big && wide) *wide = 1;
     __syncthreads();
     for (int r = b; r < 32; r += 8)
       if (i0 + r < N && j0 + a < count) v[size_t(i0 + r) * Cp + column(q0 + j0 + a)] = t[r][a];

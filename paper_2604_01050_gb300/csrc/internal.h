@@ -351,8 +351,8 @@ cudaError_t launch_solve_batched(const SlotDesc *slots, int n_slots, const WorkI
                                  int grid, int j0, int j1, unsigned *bar, int *err, cudaStream_t st);
 
 // Replicas q0 .. q0 + count - 1 (run-major) of the state array v [N][Cp] to
-// (out) or from rows [count][N]; *wide becomes 1 when a value read is not
-// below 2 in magnitude (init_readout.cu).
+// (out) or from rows [count][N]; *wide (unless null) becomes 1 when a value
+// read is not below 2 in magnitude (init_readout.cu).
 cudaError_t launch_state_rows(const StateView &s, float *v, float *rows, int q0, int count, bool out, int *wide,
                               cudaStream_t st);
 int energy_row_blocks(int N);

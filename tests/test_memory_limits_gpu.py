@@ -76,3 +76,40 @@ def test_a_run_that_does_not_fit_without_the_planes_either(sb, monkeypatch):
     assert e.value.status == sb.ERR_OOM
     sb.run(pb, 30, 8, 128, seed=2)
     assert np.isfinite(sb.get_best(pb)["energy"]).all()
+
+
+@pytest.mark.parametrize("N,P,R", [(1, 1, 200), (3, 7, 60), (33, 12, 40), (500, 3, 50)])
+@pytest.mark.parametrize("variant", ["threshold", "ballistic"])
+def test_state_transfers_without_a_slice(sb, monkeypatch, N, P, R, variant):
+    """No memory for the slice that state transfers pass through: get_state and set_state work as before,
+    in several slices, and the run goes on the same way; a state outside the wall is still seen."""
+    up = np.triu(np.random.default_rng(N).standard_normal((N, N)), 1)
+    J = up + up.T
+    rows, cols = np.nonzero(J)
+    if variant == "ballistic":  # sparse, a ring, for the form that looks at the state's range
+        rows = np.repeat(np.arange(N), 2) if N > 2 else np.zeros(0, int)
+        cols = np.sort(np.stack([np.arange(N) - 1, np.arange(N) + 1], 1) % N, axis=1).ravel() if N > 2 else rows
+    rp = np.concatenate([[0], np.cumsum(np.bincount(rows, minlength=N))])
+    val = np.ones(rows.size) if variant == "ballistic" else J[rows, cols]
+    out = []
+    for fail in (False, True):
+        pb = sb.create_problem_csr(N, rp, cols, val)
+        sb.set_schedule(pb, precision="fp32", variant=variant, gamma0=4.0 * P, kernel_select=2)
+        sb.run_begin(pb, 12, P, R, seed=3)
+        sb.run_advance(pb, 5)
+        if fail:
+            monkeypatch.setenv("SBQA_TEST_FAIL_ALLOC", "1:1000")
+        x, y, done = sb.get_state(pb)
+        x[R - 1, P - 1, N - 1] = 2.5
+        y[0, 0, 0] = -3.0
+        sb.set_state(pb, x, y, done)
+        x2, y2, _ = sb.get_state(pb)
+        assert np.array_equal(x, x2) and np.array_equal(y, y2)
+        kernel = pb.info().step_kernel
+        monkeypatch.delenv("SBQA_TEST_FAIL_ALLOC", raising=False)
+        sb.run_advance(pb, 7)
+        sb.run_finish(pb)
+        out.append((x, y, kernel, *sb.get_state(pb)[:2], sb.get_best(pb)["spins"]))
+    assert all(np.array_equal(a, b) for a, b in zip(*out))
+    if variant == "ballistic":
+        assert out[0][2] == 6
