@@ -130,7 +130,8 @@ __global__ void __launch_bounds__(kFxThreads, 1)
   uint64_t *full = reinterpret_cast<uint64_t *>(cols + 4 * kTcBN * 2);
   uint64_t *empty = full + kFxStages;
   uint64_t *acc_full = empty + kFxStages, *acc_free = acc_full + 2;
-  uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(acc_free + 2);
+  uint64_t *drained = acc_free + 2;
+  uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(drained + 1);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int m0 = blockIdx.y * kTcBM, n0 = blockIdx.x * kTcBN;
   const int KB = Kp / 64, total = KB * kFxDigits;
@@ -143,6 +144,7 @@ __global__ void __launch_bounds__(kFxThreads, 1)
       tc::mbar_init(&acc_full[q], 1);
       tc::mbar_init(&acc_free[q], 16);
     }
+    tc::mbar_init(drained, 1);
     tc::fence_mbar_init();
     tc::prefetch_tmap(&mapA);
     tc::prefetch_tmap(&mapB);
@@ -154,14 +156,19 @@ __global__ void __launch_bounds__(kFxThreads, 1)
   const uint32_t tmem = *tmem_slot;
   uint64_t acc[32];
   if (warp == 16) {
-    if (lane == 0)
-      for (int g = 0; g < total; ++g) {
+    if (lane == 0) {
+      int g = 0;
+      for (; g < total; ++g) {
         const int st = g % kFxStages, use = g / kFxStages, d = g / KB, kb = g % KB;
         if (use > 0 && !tc::mbar_wait(&empty[st], (use - 1) & 1, err, tc::ERR_WAIT_EMPTY)) break;
         tc::mbar_arrive_expect_tx(&full[st], 2 * kTcTile);
         tc::tma_load_2d(sA + st * kTcTile, &mapA, &full[st], kb * 64, d * Kp + m0);
         tc::tma_load_2d(sB + st * kTcTile, &mapB, &full[st], kb * 64, n0);
       }
+      // no copy lands once the stages are reused, whether the MMAs took them or a wait ran out
+      for (int q = max(0, g - kFxStages); q < g; ++q)
+        tc::mbar_wait(&full[q % kFxStages], (q / kFxStages) & 1, err, tc::ERR_WAIT_FULL);
+    }
   } else if (warp == 17) {
     if (lane == 0) {
       constexpr uint32_t idesc = tc::idesc_bf16(kTcBM, kTcBN);
@@ -183,6 +190,10 @@ __global__ void __launch_bounds__(kFxThreads, 1)
         }
         if (ok) tc::mma_commit(&acc_full[d & 1]);
       }
+      if (!ok) {  // the epilogue has not waited for these
+        tc::mma_commit(drained);
+        tc::mbar_wait(drained, 0, err, tc::ERR_WAIT_DONE);
+      }
     }
   } else {
     const uint32_t at = tmem + (uint32_t((warp & 3) * 32) << 16) + uint32_t(32 * (warp >> 2));
@@ -203,8 +214,7 @@ __global__ void __launch_bounds__(kFxThreads, 1)
         acc[j] = (acc[j] << 8) + uint64_t(int64_t(__float2int_rn(__uint_as_float(g[j]))));
     }
   }
-  // every MMA that read the stages has completed once the last digit is in (or the run has failed):
-  // row reductions reuse them
+  // every copy into the stages and every MMA that read them has completed: row reductions reuse them
   __syncthreads();
   if (warp < 16) {
     const int quarter = warp & 3, chunk = warp >> 2;
