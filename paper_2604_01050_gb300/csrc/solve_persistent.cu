@@ -821,6 +821,13 @@ static int cache_cap_hook() {
   return k > 0 ? k : (1 << 30);
 }
 
+// Test hook: SBQA_TEST_PERSIST_PASSES=k sends run batches of more than k passes per warp to the streaming
+// form, so that small instances take it (not for production use).
+static int max_passes() {
+  const char *v = std::getenv("SBQA_TEST_PERSIST_PASSES");
+  return v ? std::max(0, std::min(kMaxPasses, std::atoi(v))) : kMaxPasses;
+}
+
 // Blocks of the grid: one per SM, as the registers and shared memory of every
 // instantiation allow (0 when one does not fit the device, or the streaming
 // form's blocks do not).  Also sets their shared-memory limits, which last for
@@ -861,7 +868,7 @@ static void split_smem(PersistArgs *a, long long units, int warps, int eb, int p
 // L = 24: 61 items, 126 against 119).
 static bool bsb_resident(int N, int Cp, int blocks) {
   return (long long)N * (Cp / kColsPerWarp) <=
-         (long long)blocks * kPersistWarps * std::min(kMaxPasses, cache_cap_hook());
+         (long long)blocks * kPersistWarps * std::min(max_passes(), cache_cap_hook());
 }
 
 bool persistent_bsb_ok(int N, int Cp, int max_degree, int kind, int blocks) {
@@ -924,7 +931,7 @@ int persistent_mode(int N, int Cp, int max_degree, int kind, int blocks, bool fo
   const bool wide = max_degree > kPersistMaxDeg;
   if (blocks <= 0 || max_degree > kPersistWideDeg || lpi == 0 || (!wide && !ell)) return 0;
   const long long items = (long long)N * (Cp / (8 * lpi)), warps = (long long)blocks * kPersistWarps;
-  long long most = std::min<long long>(kMaxPasses * (32 / lpi), cache_cap_hook());
+  long long most = std::min<long long>(max_passes() * (32 / lpi), cache_cap_hook());
   if (wide) most = std::min<long long>(most, kWarpSmem / wide_bytes((max_degree + 3) / 4 * 4, kind != VAL_PM1));
   if (!force_rows && items <= warps * most) return kPersistResident;
   return wide ? 0 : streaming_mode(N, Cp, max_degree, kind, blocks * kStreamBlocksPerSm, force_rows, ell);
