@@ -1492,6 +1492,25 @@ struct StateSlices {
   }
 };
 
+// Small states are copied as they lie and change layout on the host: a slice,
+// its kernel and their waits cost more than the copies.  Values of the state
+// array and of the caller's, and the mean us of get_state and set_state (host /
+// device): 3456 and 27 35 / 62, 3456 and 3456 38 / 64, 27648 and 216 43 / 62,
+// 13824 and 13824 58 / 67; on the other side of the line 128000 and 1000 59 /
+// 61, 27648 and 27648 88 / 70, 128000 and 128000 302 / 74.
+bool state_on_host(const sbqa_problem *p) {
+  return size_t(p->n) * (size_t(p->Cp) + 4 * size_t(p->R) * p->P) <= size_t(72) << 10;
+}
+
+// Calls f(index in the state array, index in the caller's) for every value.
+template <class F>
+void for_state(const sbqa_problem *p, F f) {
+  for (int q = 0; q < p->R * p->P; ++q) {
+    const size_t c = size_t(q / p->P) * p->Ps + q % p->P;
+    for (int i = 0; i < p->n; ++i) f(size_t(i) * p->Cp + c, size_t(q) * p->n + i);
+  }
+}
+
 }  // namespace
 
 // ---- helpers shared with the batching engine (problem.h) ----
@@ -2152,8 +2171,20 @@ int sbqa_get_state(sbqa_problem *p, float *x, float *y, int32_t *step_done) {
   int rc = sbqa_synchronize(p);
   if (rc != SBQA_OK) return rc;
   DeviceGuard g(p->device);
-  StateSlices sl(p);
   float *outs[2] = {x, y}, *src[2] = {p->d_x.p, p->d_y.p};
+  if (state_on_host(p)) {
+    const size_t NC = size_t(p->n) * p->Cp;
+    std::vector<float> buf(2 * NC);
+    for (int w = 0; w < 2; ++w)
+      if (outs[w])
+        SBQA_CUDA(cudaMemcpyAsync(buf.data() + w * NC, src[w], NC * sizeof(float), cudaMemcpyDeviceToHost, p->stream));
+    SBQA_CUDA(cudaStreamSynchronize(p->stream));
+    for (int w = 0; w < 2; ++w)
+      if (outs[w]) for_state(p, [&](size_t dev, size_t out) { outs[w][out] = buf[w * NC + dev]; });
+    if (step_done) *step_done = p->step_done;
+    return SBQA_OK;
+  }
+  StateSlices sl(p);
   for (int w = 0; w < 2; ++w) {
     if (!outs[w]) continue;
     for (int q0 = 0; q0 < sl.replicas; q0 += sl.per_slice) {
@@ -2175,24 +2206,37 @@ int sbqa_set_state(sbqa_problem *p, const float *x, const float *y, int32_t step
   int rc = sbqa_synchronize(p);
   if (rc != SBQA_OK) return rc;
   DeviceGuard g(p->device);
-  StateSlices sl(p);
   const size_t NC = size_t(p->n) * p->Cp;
   const float *in[2] = {x, y};
   float *dst[2] = {p->d_x.p, p->d_y.p};
-  int *wide = reinterpret_cast<int *>(sl.rows + size_t(sl.per_slice) * p->n), is_wide = 0;
-  SBQA_CUDA(cudaMemsetAsync(wide, 0, sizeof(int), p->stream));
-  for (int w = 0; w < 2; ++w) {
-    SBQA_CUDA(cudaMemsetAsync(dst[w], 0, NC * sizeof(float), p->stream));  // padding columns of a run stay at zero
-    for (int q0 = 0; q0 < sl.replicas; q0 += sl.per_slice) {
-      const int count = std::min(sl.per_slice, sl.replicas - q0);
-      SBQA_CUDA(cudaMemcpyAsync(sl.rows, in[w] + size_t(q0) * p->n, size_t(count) * p->n * sizeof(float),
-                                cudaMemcpyHostToDevice, p->stream));
-      SBQA_CUDA(launch_state_rows(p->state(), dst[w], sl.rows, q0, count, false, w == 0 ? wide : nullptr, p->stream));
-      SBQA_CUDA(cudaStreamSynchronize(p->stream));
+  int is_wide = 0;
+  if (state_on_host(p)) {
+    std::vector<float> buf(2 * NC, 0.f);  // padding columns of a run stay at zero
+    for (int w = 0; w < 2; ++w) {
+      for_state(p, [&](size_t dev, size_t from) {
+        buf[w * NC + dev] = in[w][from];
+        if (w == 0 && !(std::fabs(in[w][from]) < 2.f)) is_wide = 1;
+      });
+      SBQA_CUDA(cudaMemcpyAsync(dst[w], buf.data() + w * NC, NC * sizeof(float), cudaMemcpyHostToDevice, p->stream));
     }
+    SBQA_CUDA(cudaStreamSynchronize(p->stream));
+  } else {
+    StateSlices sl(p);
+    int *wide = reinterpret_cast<int *>(sl.rows + size_t(sl.per_slice) * p->n);
+    SBQA_CUDA(cudaMemsetAsync(wide, 0, sizeof(int), p->stream));
+    for (int w = 0; w < 2; ++w) {
+      SBQA_CUDA(cudaMemsetAsync(dst[w], 0, NC * sizeof(float), p->stream));
+      for (int q0 = 0; q0 < sl.replicas; q0 += sl.per_slice) {
+        const int count = std::min(sl.per_slice, sl.replicas - q0);
+        SBQA_CUDA(cudaMemcpyAsync(sl.rows, in[w] + size_t(q0) * p->n, size_t(count) * p->n * sizeof(float),
+                                  cudaMemcpyHostToDevice, p->stream));
+        SBQA_CUDA(launch_state_rows(p->state(), dst[w], sl.rows, q0, count, false, w == 0 ? wide : nullptr, p->stream));
+        SBQA_CUDA(cudaStreamSynchronize(p->stream));
+      }
+    }
+    SBQA_CUDA(cudaMemcpyAsync(&is_wide, wide, sizeof(int), cudaMemcpyDeviceToHost, p->stream));
+    SBQA_CUDA(cudaStreamSynchronize(p->stream));
   }
-  SBQA_CUDA(cudaMemcpyAsync(&is_wide, wide, sizeof(int), cudaMemcpyDeviceToHost, p->stream));
-  SBQA_CUDA(cudaStreamSynchronize(p->stream));
   p->wide_x = is_wide != 0;
   const double tau = p->S > 0 ? double(step_done) / double(p->S) : 0.0;
   SBQA_CUDA(launch_refresh_f(p->state(), step_done & 1, float(p->prm.delta_slope * tau), p->stream));

@@ -78,7 +78,7 @@ def test_a_run_that_does_not_fit_without_the_planes_either(sb, monkeypatch):
     assert np.isfinite(sb.get_best(pb)["energy"]).all()
 
 
-@pytest.mark.parametrize("N,P,R", [(1, 1, 200), (3, 7, 60), (33, 12, 40), (500, 3, 50)])
+@pytest.mark.parametrize("N,P,R", [(1, 1, 20000), (3, 7, 1500), (33, 12, 60), (500, 3, 50)])
 @pytest.mark.parametrize("variant", ["threshold", "ballistic"])
 def test_state_transfers_without_a_slice(sb, monkeypatch, N, P, R, variant):
     """No memory for the slice that state transfers pass through: get_state and set_state work as before,
