@@ -993,7 +993,7 @@ struct TuneKey {
 struct TuneResult {
   int csr_variant = 0;
   bool use_persistent = false, use_tc_persistent = false, use_tc_split = false, use_tc_pair = false,
-       use_tc_f4 = false, use_tc_f4_pair = false;
+       use_tc_f4 = false, use_tc_f4_pair = false, bsb_streams = false;
   float variant_ms[8] = {};
   float persistent_ms = 0.f, tc_step_ms = 0.f, tc_persistent_ms = 0.f;
 };
@@ -1037,7 +1037,8 @@ cudaError_t clear_f(sbqa_problem *p) {
 
 // The ballistic form has one per-step kernel and, where the items fit the
 // cache, the persistent solver: kernel_select 1 keeps the per-step kernel, 2
-// the persistent solver, 0 times both (a few steps each) and keeps the faster.
+// the persistent solver, 0 times both (a few steps each) and keeps the faster;
+// of the persistent solver the streaming form too where it may be the faster.
 int autotune_csr_bsb(sbqa_problem *p) {
   if (p->csr_variant < 0) p->csr_variant = 0;
   const int sel = p->prm.kernel_select;
@@ -1045,7 +1046,7 @@ int autotune_csr_bsb(sbqa_problem *p) {
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
   SBQA_CUDA(cudaStreamIsCapturing(p->stream, &cs));
   if (cs != cudaStreamCaptureStatusNone) return SBQA_OK;
-  p->use_persistent = false;
+  p->use_persistent = p->bsb_streams = false;
   p->persistent_ms = 0.f;
   if (p->persist_blocks == 0) p->persist_blocks = memo_blocks(persistent_blocks);
   if (p->S > 0 && (sel == 0 || sel == 2) && p->persistent_ok()) {
@@ -1059,6 +1060,7 @@ int autotune_csr_bsb(sbqa_problem *p) {
       p->variant_ms[0] = known.variant_ms[0];
       p->persistent_ms = known.persistent_ms;
       p->use_persistent = known.use_persistent;
+      p->bsb_streams = known.bsb_streams;
     } else {
       const int reps = 8, steps = std::min(p->S, 64);
       float step_ms = 0.f;
@@ -1068,19 +1070,28 @@ int autotune_csr_bsb(sbqa_problem *p) {
       cudaEvent_t e0, e1;
       SBQA_CUDA(cudaEventCreate(&e0));
       SBQA_CUDA(cudaEventCreate(&e1));
-      cudaError_t e = clear_f(p);
-      if (e == cudaSuccess)
-        e = launch_solve_csr_persistent_bsb(s, J, p->tables, 0, std::min(p->S, 4), p->d_bar.p, p->d_err.p,
-                                            p->persist_blocks, p->stream);
-      if (e == cudaSuccess) e = clear_f(p);
-      if (e == cudaSuccess) e = cudaEventRecord(e0, p->stream);
-      if (e == cudaSuccess)
-        e = launch_solve_csr_persistent_bsb(s, J, p->tables, 0, steps, p->d_bar.p, p->d_err.p, p->persist_blocks,
-                                            p->stream);
-      if (e == cudaSuccess) e = cudaEventRecord(e1, p->stream);
-      if (e == cudaSuccess) e = cudaEventSynchronize(e1);
-      float ms = 0.f;
-      if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, e0, e1);
+      auto time_form = [&](bool streams, float *ms) {
+        auto run_steps = [&](int n) {
+          return launch_solve_csr_persistent_bsb(s, J, p->tables, 0, n, p->d_bar.p, p->d_err.p, p->persist_blocks,
+                                                 streams, p->stream);
+        };
+        cudaError_t c = clear_f(p);
+        if (c == cudaSuccess) c = run_steps(std::min(p->S, 4));
+        if (c == cudaSuccess) c = clear_f(p);
+        if (c == cudaSuccess) c = cudaEventRecord(e0, p->stream);
+        if (c == cudaSuccess) c = run_steps(steps);
+        if (c == cudaSuccess) c = cudaEventRecord(e1, p->stream);
+        if (c == cudaSuccess) c = cudaEventSynchronize(e1);
+        if (c == cudaSuccess) c = cudaEventElapsedTime(ms, e0, e1);
+        return c;
+      };
+      float ms = 0.f, streaming_ms = 0.f;
+      cudaError_t e = time_form(false, &ms);
+      if (e == cudaSuccess && persistent_bsb_may_stream(p->n, p->Cp, p->max_degree, p->kind, p->persist_blocks)) {
+        e = time_form(true, &streaming_ms);
+        p->bsb_streams = streaming_ms < ms;
+        ms = std::min(ms, streaming_ms);
+      }
       cudaEventDestroy(e0);
       cudaEventDestroy(e1);
       SBQA_CUDA(e);
@@ -1092,6 +1103,7 @@ int autotune_csr_bsb(sbqa_problem *p) {
       r.variant_ms[0] = step_ms;
       r.persistent_ms = p->persistent_ms;
       r.use_persistent = p->use_persistent;
+      r.bsb_streams = p->bsb_streams;
       tune_store(p, r);
     }
   }
@@ -1427,7 +1439,8 @@ cudaError_t issue_range(sbqa_problem *p, int n0, int n1, cudaStream_t st) {
       if (K > 0) stop = std::min(n1, (n / K + 1) * K);
       cudaError_t e = tc_persist      ? launch_tc_persistent(p, p->state(), n, stop, st)
                       : p->ballistic() ? launch_solve_csr_persistent_bsb(p->state(), p->csr(), p->tables, n, stop,
-                                                                          p->d_bar.p, p->d_err.p, p->persist_blocks, st)
+                                                                          p->d_bar.p, p->d_err.p, p->persist_blocks,
+                                                                          p->bsb_streams, st)
                                        : launch_solve_csr_persistent(p->state(), p->csr(), p->tables, n, stop,
                                                                      p->d_bar.p, p->d_err.p, p->persist_blocks,
                                                                      p->persist_mode(), st);

@@ -215,6 +215,7 @@ struct sbqa_problem {
   float variant_ms[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
   bool use_persistent = false;  // autotuner: one cooperative launch for all steps
   float persistent_ms = 0.f;    // its timing per step
+  bool bsb_streams = false;     // autotuner: the ballistic form's streaming solver, where the on-chip one fits too
   bool wide_x = false;  // sbqa_set_state gave some |x| >= 2 or NaN: ballistic runs stay on the per-step kernel
   int persist_blocks = 0;
   sbqa::DevBuf<unsigned> d_bar;  // grid barrier counters of the streaming form

@@ -864,8 +864,8 @@ static void split_smem(PersistArgs *a, long long units, int warps, int eb, int p
 }
 
 // Items of the ballistic form a warp takes at most before the streaming form
-// is the faster one (L = 20, R*P = 2048: 35 items, 70 us per step against 71;
-// L = 24: 61 items, 126 against 119).
+// is the faster one (L = 24, R*P = 2048: 61 items, 126 us per step against
+// 119).  Below, see persistent_bsb_may_stream.
 static bool bsb_resident(int N, int Cp, int blocks) {
   return (long long)N * (Cp / kColsPerWarp) <=
          (long long)blocks * kPersistWarps * std::min(max_passes(), cache_cap_hook());
@@ -874,6 +874,23 @@ static bool bsb_resident(int N, int Cp, int blocks) {
 bool persistent_bsb_ok(int N, int Cp, int max_degree, int kind, int blocks) {
   if (blocks <= 0 || max_degree > kPersistMaxDeg || Cp % kColsPerWarp != 0) return false;
   return bsb_resident(N, Cp, blocks) || streaming_bsb_ok(N, Cp, max_degree, kind, blocks * kStreamBlocksPerSm);
+}
+
+// Whether the two ballistic forms are close enough for the autotuner to time
+// both.  Bound by the ALU pipe, an item takes the on-chip form 0.78 of its time
+// in the streaming one (1.83 and 2.35 us at one block per SM), but that has 32
+// warps per SM to the 24 here, and the fullest warp sets the step: L = 14, R*P =
+// 1024, 7 items against 5: 12.9 us per step and 11.5 streaming; L = 20, R*P =
+// 2048, 36 against 27: 67.6 and 63.9; but 18 against 14, L = 16: 32.0 and 36.6.
+// Where the on-chip form has less than 5 items for 4, it was the faster one in
+// every shape measured (L = 6 .. 20, random graphs of N = 3000 .. 10^5, R*P =
+// 128 .. 2048).
+bool persistent_bsb_may_stream(int N, int Cp, int max_degree, int kind, int blocks) {
+  if (!bsb_resident(N, Cp, blocks) || !streaming_bsb_ok(N, Cp, max_degree, kind, blocks * kStreamBlocksPerSm))
+    return false;
+  const long long items = (long long)N * (Cp / kColsPerWarp), on_chip = (long long)blocks * kPersistWarps,
+                  streaming = (long long)blocks * kStreamBlocksPerSm * 8;
+  return 4 * ((items + on_chip - 1) / on_chip) >= 5 * ((items + streaming - 1) / streaming);
 }
 
 static PersistArgs persist_args(const StateView &s, const CsrView &J, const StepTables &t, int n_begin, int n_end,
@@ -916,8 +933,10 @@ static cudaError_t launch_persist(const void *fn, PersistArgs &a, int kind, void
 }
 
 cudaError_t launch_solve_csr_persistent_bsb(const StateView &s, const CsrView &J, const StepTables &t, int n_begin,
-                                            int n_end, unsigned *bar, int *err, int blocks, cudaStream_t st) {
-  if (!bsb_resident(s.N, s.Cp, blocks))
+                                            int n_end, unsigned *bar, int *err, int blocks, bool streams,
+                                            cudaStream_t st) {
+  if ((streams && streaming_bsb_ok(s.N, s.Cp, J.max_degree, J.kind, blocks * kStreamBlocksPerSm)) ||
+      !bsb_resident(s.N, s.Cp, blocks))
     return launch_solve_csr_streaming_bsb(s, J, t, n_begin, n_end, bar, err, blocks * kStreamBlocksPerSm, st);
   PersistArgs a = persist_args(s, J, t, n_begin, n_end, err);
   split_smem(&a, (long long)s.N * (s.Cp / kColsPerWarp), blocks * kPersistWarps, entry_bytes(J.kind != VAL_PM1), 1,

@@ -90,3 +90,13 @@ def test_a_wait_that_runs_out_is_reported_and_the_handle_recovers(sb, monkeypatc
     monkeypatch.delenv("SBQA_TEST_SKIP_BARRIER_STEP")
     _solve(sb, spec, 8, 16, 40, 2, pb=pb, **kw)
     _equal(sb, _solve(sb, spec, 8, 16, 40, 1, **kw), pb)
+
+
+@pytest.mark.parametrize("L,P,R", [(14, 16, 64), (14, 7, 128), (16, 16, 128), (20, 8, 48)])
+def test_the_ballistic_form_the_autotuner_keeps(sb, L, P, R):
+    """Shapes where it times the on-chip form and the streaming one."""
+    _, spec = lattice(L, 3)
+    kw = dict(variant="ballistic", gamma0=4.0 * P, eval_every=13)
+    a, b = (_solve(sb, spec, P, R, 30, ks, **kw) for ks in (1, 0))
+    assert b.info().step_kernel == 14 and 0 < b.info().persistent_ms < b.info().variant_ms[0]
+    _equal(sb, a, b)
