@@ -136,8 +136,10 @@ cudaError_t launch_solve_csr_streaming_bsb(const StateView &s, const CsrView &J,
 // cached per warp; f buffers Fx in FP32): eligible when the items fit the
 // cache (persistent_bsb_ok); results equal launch_step_csr_bsb bit for bit.
 // streams: the streaming form also where the on-chip one is the rule
-// (persistent_bsb_may_stream: both are worth timing).
+// (persistent_bsb_may_stream: both are worth timing; persistent_bsb_streams:
+// which one a launch takes).
 bool persistent_bsb_ok(int N, int Cp, int max_degree, int kind, int blocks);
+bool persistent_bsb_streams(int N, int Cp, int max_degree, int kind, int blocks, bool wanted);
 bool persistent_bsb_may_stream(int N, int Cp, int max_degree, int kind, int blocks);
 cudaError_t launch_solve_csr_persistent_bsb(const StateView &s, const CsrView &J, const StepTables &t, int n_begin,
                                             int n_end, unsigned *bar, int *err, int blocks, bool streams,

@@ -216,7 +216,7 @@ struct sbqa_problem {
   bool use_persistent = false;  // autotuner: one cooperative launch for all steps
   float persistent_ms = 0.f;    // its timing per step
   bool bsb_streams = false;     // autotuner: the ballistic form's streaming solver, where the on-chip one fits too
-  bool wide_x = false;  // sbqa_set_state gave some |x| >= 2 or NaN: ballistic runs stay on the per-step kernel
+  bool wide_x = false;  // sbqa_set_state gave some |x| >= 2 or NaN: not for the on-chip ballistic solver
   int persist_blocks = 0;
   sbqa::DevBuf<unsigned> d_bar;  // grid barrier counters of the streaming form
   int csr_variant_cp = -1, csr_variant_kind = -1, csr_variant_select = -1;
@@ -327,7 +327,10 @@ struct sbqa_problem {
 
   bool persistent_ok() const {
     if (dense) return false;
-    if (ballistic()) return !wide_x && sbqa::persistent_bsb_ok(n, Cp, max_degree, kind, persist_blocks);
+    if (ballistic()) {
+      return sbqa::persistent_bsb_ok(n, Cp, max_degree, kind, persist_blocks) &&
+             (!wide_x || sbqa::persistent_bsb_streams(n, Cp, max_degree, kind, persist_blocks, bsb_streams));
+    }
     return persist_mode() != 0;
   }
 

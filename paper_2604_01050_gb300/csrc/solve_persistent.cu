@@ -893,6 +893,11 @@ bool persistent_bsb_may_stream(int N, int Cp, int max_degree, int kind, int bloc
   return 4 * ((items + on_chip - 1) / on_chip) >= 5 * ((items + streaming - 1) / streaming);
 }
 
+bool persistent_bsb_streams(int N, int Cp, int max_degree, int kind, int blocks, bool wanted) {
+  return !bsb_resident(N, Cp, blocks) ||
+         (wanted && streaming_bsb_ok(N, Cp, max_degree, kind, blocks * kStreamBlocksPerSm));
+}
+
 static PersistArgs persist_args(const StateView &s, const CsrView &J, const StepTables &t, int n_begin, int n_end,
                                 int *err) {
   PersistArgs a;
@@ -935,8 +940,7 @@ static cudaError_t launch_persist(const void *fn, PersistArgs &a, int kind, void
 cudaError_t launch_solve_csr_persistent_bsb(const StateView &s, const CsrView &J, const StepTables &t, int n_begin,
                                             int n_end, unsigned *bar, int *err, int blocks, bool streams,
                                             cudaStream_t st) {
-  if ((streams && streaming_bsb_ok(s.N, s.Cp, J.max_degree, J.kind, blocks * kStreamBlocksPerSm)) ||
-      !bsb_resident(s.N, s.Cp, blocks))
+  if (persistent_bsb_streams(s.N, s.Cp, J.max_degree, J.kind, blocks, streams))
     return launch_solve_csr_streaming_bsb(s, J, t, n_begin, n_end, bar, err, blocks * kStreamBlocksPerSm, st);
   PersistArgs a = persist_args(s, J, t, n_begin, n_end, err);
   split_smem(&a, (long long)s.N * (s.Cp / kColsPerWarp), blocks * kPersistWarps, entry_bytes(J.kind != VAL_PM1), 1,

@@ -100,3 +100,24 @@ def test_the_ballistic_form_the_autotuner_keeps(sb, L, P, R):
     a, b = (_solve(sb, spec, P, R, 30, ks, **kw) for ks in (1, 0))
     assert b.info().step_kernel == 14 and 0 < b.info().persistent_ms < b.info().variant_ms[0]
     _equal(sb, a, b)
+
+
+@pytest.mark.parametrize("value", [2.5, -7.0, np.inf, np.nan])
+def test_streaming_takes_states_from_outside_the_wall(sb, monkeypatch, value):
+    """The streaming ballistic solver has no bit to spare in a position: it takes any state, as the
+    per-step kernel does."""
+    _, spec = lattice(6, 8)
+    P, R, steps = 4, 8, 12
+    monkeypatch.setenv("SBQA_TEST_PERSIST_PASSES", "0")
+    out = []
+    for ks in (1, 2):
+        pb = create(sb, spec)
+        sb.set_schedule(pb, *workloads.autotune_params(R, 2), kernel_select=ks, variant="ballistic", gamma0=16.0)
+        sb.run_begin(pb, steps, P, R, seed=3)
+        x, y, _ = sb.get_state(pb)
+        x[1, 2, 5] = value
+        sb.set_state(pb, x, y, 0)
+        sb.run_advance(pb, steps)
+        assert pb.info().step_kernel == (14 if ks == 2 else 6)
+        out.append(sb.get_state(pb))
+    assert np.array_equal(out[0][0], out[1][0]) and np.array_equal(out[0][1], out[1][1])
