@@ -748,7 +748,7 @@ def gpu_context():
 
 KERNEL_NAMES = {0: "k_step_csr", 1: "k_step_dense", 2: "k_step_dense_tc", 3: "k_solve_small",
                 4: "k_solve_csr_persistent", 5: "k_solve_dense_tc_persistent", 6: "k_step_csr_bsb",
-                7: "k_step_dense_bsb", 8: "k_solve_dense_tc_split", 9: "k_solve_dense_tc_pair",
+                7: "k_step_dense<ballistic>", 8: "k_solve_dense_tc_split", 9: "k_solve_dense_tc_pair",
                 10: "k_step_dense_tc<bf16>", 11: "k_solve_dense_tc_persistent<bf16>",
                 12: "k_step_dense_tc<bsb>", 13: "k_solve_dense_tc_persistent<bsb>", 14: "k_solve_csr_persistent_bsb",
                 15: "k_solve_dense_tc_f4", 16: "k_solve_dense_tc_f4_pair"}
@@ -818,12 +818,20 @@ def roofline_of(cfg, name, info, N, P, R, step_ms, peaks):
     bpu = BYTES_PER_UPDATE_BSB if info.step_kernel in (6, 7, 14) else BYTES_PER_UPDATE
     achieved_gbs = bpu * N * P * R / (step_ms * 1e-3) / 1e9
     hbm_peak = peaks.get("hbm_gbs", 6800.0)
-    return {"bound": "hbm", "achieved": achieved_gbs, "peak": hbm_peak, "unit": "GB/s",
-            "frac": achieved_gbs / hbm_peak, "traffic": traffic, "kernel": kname, "step_ms": step_ms,
-            "peak_source": peak_src,
-            "note": "algorithmic %d B/update x N*P*R per launch / event-timed step time" % bpu +
-                    ("; x and y stay on the chip between steps where they fit, so this can exceed the HBM peak"
-                     if info.step_kernel in (4, 14) else "")}
+    rec = {"bound": "hbm", "achieved": achieved_gbs, "peak": hbm_peak, "unit": "GB/s",
+           "frac": achieved_gbs / hbm_peak, "traffic": traffic, "kernel": kname, "step_ms": step_ms,
+           "peak_source": peak_src,
+           "note": "algorithmic %d B/update x N*P*R per launch / event-timed step time" % bpu}
+    if info.step_kernel in (4, 14):  # the persistent CSR solvers: what of it moves, and the arithmetic
+        rec["note"] += "; x and y stay on the chip between steps where they fit, so this is no roofline of the " \
+                       "on-chip form and can exceed the HBM peak: see traffic_frac (the captured DRAM bytes over " \
+                       "the step time) and fp32_frac (2 flops a coupling + 14 an update, of the derived FP32 rate)"
+        if traffic is not None:
+            rec["traffic_frac"] = traffic / (step_ms * 1e-3) / 1e9 / hbm_peak
+        if getattr(info, "nnz", 0):
+            flops = (2.0 * info.nnz + 14.0 * N) * P * R
+            rec["fp32_frac"] = flops / (step_ms * 1e-3) / (152 * 128 * 2 * peaks.get("sm_max_mhz", 2070.0) * 1e6)
+    return rec
 
 
 def measure_config(name, cfg, args, ctx, cpu_seconds):

@@ -344,7 +344,10 @@ cudaError_t launch_energy_dense_fx(const StateView &s, const EnergyView &E, void
 // on ties; replica k of run r is column r * P + k), kept if strictly lower
 // than the best so far; then all threads copy the winner's spins (a strided
 // gather of N bytes).  From N = kBestSplit on the copy is a kernel of its own
-// over blocks of spins (N = 10^5, 8 runs: 190 us by 8 blocks).
+// over blocks of spins.  A readout, us, in one kernel / with the copy on its own:
+// N = 2048 27.8 / 30.9 (R*P = 128), 4096 31.4 / 31.4, 8192 44.5 / 39.6, 16384
+// 66.2 / 56.2, 32768 106.7 / 82.6, 10^5 287 / 206; R*P = 2048: 4096 136 / 136,
+// 16384 473 / 464, 32768 954 / 901.  So the line could lie at 8192 as well.
 constexpr int kBestThreads = 256, kBestSplit = 16384;
 // have_best of a run: none yet (0), from an earlier readout, or from the last one
 constexpr int kBestKept = 1, kBestNew = 2;

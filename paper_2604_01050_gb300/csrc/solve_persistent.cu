@@ -1,31 +1,38 @@
 // solve_persistent.cu -- all steps of a CSR run batch in one cooperative launch.
 //
 // For rows of degree <= 32 (+-1, FP32 or BF16 couplings; up to 8 for the
-// ballistic form, whose lists and the streaming form's are of 8 slots).  One block of 32
-// warps per SM; every warp owns fixed work items (spin row, 128 or 256
-// replica columns) for the whole launch -- individual items, or whole rows
-// with all their chunks when the items outnumber the cache.  A pass is what
+// ballistic form, whose lists and the streaming form's are of 8 slots).  One
+// block of kPersistWarps (24) warps per SM; every warp owns fixed work items
+// (spin row, 128 or 256 replica columns) for the whole launch.  A pass is what
 // the warp works on at a time: one 256-column item, or two 128-column ones on
 // its half warps (8 columns per lane either way).
 //
 // What a launch reads from memory more than once it keeps on the SM:
 //   neighbour lists (columns, signs or values, degrees) in shared memory;
-//   x and y of a warp's first passes in tensor memory (the block takes all
-//   512 TMEM columns; 64 per warp hold 4 passes of 8 + 8 values per lane) and
-//   of the next passes in the shared memory the lists leave (2 KB each).
+//   x and y of a warp's first kTmemPasses (5) passes in tensor memory (the
+//   block takes all 512 TMEM columns; the kWarpTmem = 80 of a warp hold 5
+//   passes of 8 + 8 values per lane) and of kMaxSlots (1) more in shared
+//   memory (2 KB).
 // Passes past those keep x and y in global memory, so a launch of any size
-// streams only the part of its state that does not fit the chip.  The 152
-// SMs hold 38 MB of state in TMEM and up to 31 MB in shared memory: all of the
-// 67 MB of the L = 16 lattice with R*P = 2048, 58 % of the 102 MB of N = 10^5
-// with R*P = 128.  Between SMs only the one-byte f codes move, through L2
-// (ld.global.cg: other blocks wrote them).
+// streams only the part of its state that does not fit the chip.  The 3648
+// warps of 152 SMs hold 37 MB of state in TMEM and 7.5 MB in shared memory: 6
+// of the 9 passes (67 MB) of the L = 16 lattice with R*P = 2048, whose other
+// passes stay in L2, and 6 of the 14 (102 MB) of N = 10^5 with R*P = 128.
+// Between SMs only the one-byte f codes move, through L2 (relaxed accesses at GPU
+// scope: other blocks read and write them).
 //
 // What bounds a pass then is the ALU pipe (compares, selects, logic, byte
-// permutes at half rate: about 150 a pass) and the latency of the gathers; 24
-// warps of 80 registers were faster than 32 of 64, which spill (lattice L = 16
-// 13.3 against 16.1 us per step), and one 2 KB state slot per warp faster than
-// more, which take the L1 the gathers pass through (14.5 with three, 17.4 with
-// four).  us per step, before (the streaming form) and with this kernel:
+// permutes at half rate: about 150 a pass; busy 69 % of the cycles at L = 16,
+// 63 % at degree 20, 75 % in the ballistic form) and the latency of the
+// gathers; 24 warps of 80 registers were faster than 32 of 64, which spill much
+// more (lattice L = 16 13.3 against 16.1 us per step), and one 2 KB state slot
+// per warp faster than more, which take the L1 the gathers pass through (14.5
+// with three, 17.4 with four).  At 80 registers the short lists of +-1 and real
+// J do not spill for P = 2, 4 and 16 up (P = 1: at most 12 bytes, P = 8: 4 to 36),
+// the ballistic form spills 4 to 16 bytes, and the long lists 12 to 60 but for
+// those of real J on half warps from P = 16 up, which do not; at P = 8 260 to 460
+// bytes: a general and a plain ring stand side by side.
+// us per step, before (the streaming form) and with this kernel:
 //   lattice L = 16, R*P = 2048     24.0 -> 13.3    random graph N = 10^5,
 //   lattice L = 10, R*P = 1024      4.9 ->  3.1    R*P = 128, BF16 46.8 -> 27.8
 //   lattice L = 24, R*P = 2048     81.9 -> 70.2    N = 3000 3.0 -> 2.0
@@ -64,7 +71,7 @@ namespace sbqa {
 
 constexpr int kPersistMaxDeg = 8;    // slots of the short lists
 constexpr int kPersistWideDeg = 32;  // and of the long ones
-constexpr int kWideAtOnce = 12;      // slots of a long list gathered at a time (24 registers of codes; 32 spill)
+constexpr int kWideAtOnce = 12;      // slots of a long list gathered at a time (24 registers of codes; 16 and 24 spill more)
 constexpr int kPersistWarps = 24, kPersistThreads = 32 * kPersistWarps;
 constexpr int kPersistSmem = 225 * 1024;               // dynamic shared memory of a block
 constexpr int kWarpSmem = kPersistSmem / kPersistWarps;  // 9600 bytes per warp
@@ -589,8 +596,8 @@ __global__ void __launch_bounds__(kPersistThreads, 1) k_solve_csr_persistent(Per
 // scheme with items of 128 columns on whole warps (4 columns per lane),
 // gathering the neighbours' FP32 positions of the step before (written by
 // other blocks: read through L2).  An item's own x is its entry of that f
-// buffer, so only y is separate state: it stays in TMEM for a warp's first 16
-// items and in shared memory for the next ones (512 bytes each), and x goes
+// buffer, so only y is separate state: it stays in TMEM for a warp's first 20
+// items and in shared memory for one more (512 bytes), and x goes
 // to the state array once, after the last step.  The sum runs over the row's
 // cache slots in order, a zero weight past the degree -- the sequence of
 // fused multiply-adds of k_step_csr_bsb -- and the update is sb_advance4_bsb,

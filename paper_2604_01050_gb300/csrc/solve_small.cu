@@ -287,8 +287,9 @@ __global__ void __launch_bounds__(1024) k_solve_small_i8(SmallArgs a) {
   if (live && k == kb) a.best_spins[size_t(r) * N + i] = x >= 0.f ? 1 : -1;
 }
 
-// Shared memory of the byte form; smaller than small_smem_bytes, so whatever
-// is eligible fits.
+// Shared memory of the byte form: at most 3 KB more than small_smem_bytes (N <
+// 28, where its rows are padded most), which small_eligible keeps 27 KB below
+// what a block can have.
 template <int P, int NQ>
 static cudaError_t launch_small_i8(const SmallArgs &a, cudaStream_t st) {
   const size_t smem = size_t(2) * P * (16 * NQ + 16) + size_t(a.N) * P * 8 + 8 * (P + 1) + (3 * size_t(a.S) + 1) * 4;
