@@ -74,7 +74,7 @@ struct DevBuf {
   T *p = nullptr;
   size_t n = 0;      // elements the block holds (at least the count asked for)
   size_t bytes = 0;  // its size class
-  uint64_t moves = 0;  // blocks taken so far: the address is the same while this is
+  uint64_t moves = 0;  // blocks taken and given back so far: the block is the same while this is
   cudaError_t alloc(size_t count) {
     if (count <= n && p) return cudaSuccess;
     release();
@@ -95,6 +95,7 @@ struct DevBuf {
     if (p) {
       if (!idle) cudaDeviceSynchronize();
       devcache_put(p, bytes);
+      ++moves;
     }
     p = nullptr;
     n = 0;
@@ -270,7 +271,7 @@ struct sbqa_problem {
     }
   } graph_key;
 
-  // Grows whenever a buffer that a launch may name has moved.  A graph names them all, and they move one
+  // Grows whenever a buffer that a launch may name has moved or gone.  A graph names them all, and they move one
   // by one: each keeps its block while the new size fits the block's size class.
   uint64_t buffer_moves() const {
     auto sum = [](const auto &...b) { return (uint64_t(0) + ... + b.moves); };

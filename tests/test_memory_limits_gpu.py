@@ -113,3 +113,22 @@ def test_state_transfers_without_a_slice(sb, monkeypatch, N, P, R, variant):
     assert all(np.array_equal(a, b) for a, b in zip(*out))
     if variant == "ballistic":
         assert out[0][2] == 6
+
+
+def test_the_kept_graph_after_the_planes_were_given_up(sb, monkeypatch):
+    """A run of the other form asks for buffers of its own and does not get them, with the planes or
+    without; no buffer of the first form has moved.  Its kept graph names the planes and is not used."""
+    pb = _gauss(sb, 640, gamma0=32.0)
+    sb.run(pb, 30, 8, 16, seed=2)
+    a, ea = sb.get_best(pb), sb.get_energies(pb)[0]
+    sb.set_schedule(pb, precision="fp32", gamma0=32.0, variant="ballistic")
+    monkeypatch.setenv("SBQA_TEST_FAIL_ALLOC", "100:2")
+    with pytest.raises(sb.SBQAError) as e:
+        sb.run(pb, 30, 8, 16, seed=2)
+    assert e.value.status == sb.ERR_OOM
+    monkeypatch.delenv("SBQA_TEST_FAIL_ALLOC")
+    sb.set_schedule(pb, precision="fp32", gamma0=32.0)
+    sb.run(pb, 30, 8, 16, seed=2)
+    b, eb = sb.get_best(pb), sb.get_energies(pb)[0]
+    assert np.array_equal(a["spins"], b["spins"])
+    assert np.allclose(ea, eb, rtol=1e-12, atol=1e-9) and not np.array_equal(ea, eb)
