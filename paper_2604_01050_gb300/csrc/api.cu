@@ -909,7 +909,7 @@ int alloc_run(sbqa_problem *p, int S, int P, int R) {
 int build_tables(sbqa_problem *p) {
   sbqa_problem::TablesKey key;
   key.S = p->S; key.P = p->P; key.R = p->R; key.version = p->params_version;
-  key.ka = p->d_ka.p; key.dl = p->d_dl.p; key.kj = p->d_kj.p;
+  key.moves = p->d_ka.moves + p->d_dl.moves + p->d_kj.moves;
   if (key == p->tables_key) return SBQA_OK;
   const int rc = problem_build_tables(p, p->S, p->P, p->R, p->d_ka.p, p->d_dl.p, p->d_kj.p, &p->tables, p->stream);
   p->tables_key = rc == SBQA_OK ? key : sbqa_problem::TablesKey{};

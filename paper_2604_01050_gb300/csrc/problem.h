@@ -195,10 +195,9 @@ struct sbqa_problem {
   // the schedule tables on the device were built for this (S, P, R, schedule, buffers)
   struct TablesKey {
     int S = -1, P = -1, R = -1;
-    uint64_t version = 0;
-    const void *ka = nullptr, *dl = nullptr, *kj = nullptr;
+    uint64_t version = 0, moves = 0;  // moves: of the three buffers, not their addresses, which can come back
     bool operator==(const TablesKey &o) const {
-      return S == o.S && P == o.P && R == o.R && version == o.version && ka == o.ka && dl == o.dl && kj == o.kj;
+      return S == o.S && P == o.P && R == o.R && version == o.version && moves == o.moves;
     }
   } tables_key;
   sbqa_params prm{};

@@ -55,3 +55,27 @@ def test_a_solve_after_another_operand_form(sb):
     again = sb.get_best(pb)
     for k in first:
         assert np.array_equal(first[k], again[k]), k
+
+
+def test_schedule_tables_that_came_back_to_their_old_block(sb, monkeypatch):
+    """A run that does not get memory for larger tables leaves the handle without them; another handle
+    uses their old block and returns it.  The first shape's tables lie there again, and are made again."""
+    rng = np.random.default_rng(40)
+    up = np.triu(rng.standard_normal((40, 40)), 1)
+    pb, other = (sb.create_problem_dense(up + up.T) for _ in range(2))
+    sb.set_schedule(pb, precision="fp32", gamma0=1.0)
+    sb.set_schedule(other, precision="fp32", gamma0=30.0)
+    sb.release_cached_memory()
+    sb.run(pb, 1000, 1, 250, seed=3)  # tables of 1000 x 250 entries: 1 MB
+    first = sb.get_best(pb)
+    monkeypatch.setenv("SBQA_TEST_FAIL_ALLOC", "1150000:1")
+    with pytest.raises(sb.SBQAError):
+        sb.run(pb, 1000, 1, 300, seed=3)
+    monkeypatch.delenv("SBQA_TEST_FAIL_ALLOC")
+    sb.run(other, 1000, 1, 250, seed=3)
+    sb.get_best(other)
+    other.destroy()
+    sb.run(pb, 1000, 1, 250, seed=3)
+    again = sb.get_best(pb)
+    for k in first:
+        assert np.array_equal(first[k], again[k]), k
